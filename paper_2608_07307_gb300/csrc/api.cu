@@ -75,6 +75,8 @@ struct srp_ctx {
     size_t qstate_cap = 0;
     unsigned *pix_cand = nullptr;
     size_t pix_cand_cap = 0;
+    unsigned *pix_over = nullptr;
+    size_t pix_over_cap = 0;
     int4 *big = nullptr;
     size_t big_cap = 0;
     unsigned *big_count = nullptr;
@@ -609,6 +611,7 @@ srp_status eval_plan(srp_ctx *ctx, Mesh *m, const srp_eval_params *prm, int n, b
     if (!(prm->flags & SRP_EVAL_TRAVERSE)) {
         CK(ctx, grow(&ctx->pix_key, &ctx->pix_key_cap, SL * pl.R, false));
         CK(ctx, grow(&ctx->pix_cand, &ctx->pix_cand_cap, SL * pl.R * kPixCand, false));
+        CK(ctx, grow(&ctx->pix_over, &ctx->pix_over_cap, SL * kOverWords, false));
         CK(ctx, grow(&ctx->big, &ctx->big_cap, (size_t)pl.lanes * pl.S * kBigPerSlot, false));
         CK(ctx, grow_fill(&ctx->big_count, &ctx->big_count_cap, (size_t)kLanes, 0));
         CK(ctx, grow(&ctx->bigt, &ctx->bigt_cap, (size_t)pl.lanes * pl.S * kBigPerSlot, false));
@@ -703,6 +706,7 @@ srp_status eval_enqueue(srp_ctx *ctx, Mesh *m, const srp_eval_params *prm, const
             a.rast_tris = h_tris;
             a.pix_key = ctx->pix_key + s0 * R;
             a.pix_cand = ctx->pix_cand + s0 * R * kPixCand;
+            a.pix_over = ctx->pix_over + s0 * kOverWords;
             a.big_cap = S * kBigPerSlot;
             a.big = ctx->big + (size_t)b * a.big_cap;
             a.big_count = ctx->big_count + b;
@@ -716,6 +720,7 @@ srp_status eval_enqueue(srp_ctx *ctx, Mesh *m, const srp_eval_params *prm, const
                 a.qstate = ctx->qstate + (size_t)b * qstate_words(S);
             }
         }
+        if (few_trace(Sc, R, nseg, a.raster != 0, h_tris) && !a.queue) a.few_tiles = Sc * nbx;
         int32_t *stage = ctx->hits ? ctx->hits + s0 * R * nseg : nullptr;
         a.hits = hit_tri ? (h_dev ? hit_tri + (size_t)e0 * R * nseg : stage) : ((adj || prm->n_diffuse > 0) ? stage : nullptr);
         a.walk_limit_test = (prm->flags & SRP_EVAL_TEST_WALK_BOUND) ? 1 : 0;
@@ -1016,6 +1021,7 @@ void srp_destroy(srp_ctx *ctx)
     dfree(ctx->pix_key);
     dfree(ctx->qstate);
     dfree(ctx->pix_cand);
+    dfree(ctx->pix_over);
     dfree(ctx->big);
     dfree(ctx->big_count);
     dfree(ctx->bigt);
@@ -1379,7 +1385,8 @@ srp_status srp_mesh_load(srp_ctx *ctx, const srp_mesh_desc *D, int32_t *mesh_id)
             PartInfo &pi = h.part[p];
             pi.dyn_node_off = pi.dynamic ? pi.node_begin - h.n_static_nodes : 0;
         }
-        if (3 * depth4 + 1 > kStack) {
+        h.stack_need = 3 * depth4 + 1;
+        if (h.stack_need > kStack) {
             free_tmp();
             free_mesh(m);
             return fail(ctx, SRP_ERR_MESH, "4-wide BVH depth %d exceeds the traversal stack (%d)", depth4, kStack);
@@ -2261,7 +2268,7 @@ srp_status srp_propagate_batch(srp_ctx *ctx, const srp_prop_params *p, int32_t n
     unsigned *rticket;
     int *alist, *acount, *rbad;
     unsigned long long *pkey;
-    unsigned *pcand, *bcount, *pcnt_blk;
+    unsigned *pcand, *pover, *bcount, *pcnt_blk;
     int4 *blist;
     int2 *btlist;
     SlotDesc *sd;
@@ -2296,6 +2303,7 @@ srp_status srp_propagate_batch(srp_ctx *ctx, const srp_prop_params *p, int32_t n
     CK(ctx, dmalloc(owned, &S, (size_t)n));
     CK(ctx, dmalloc(owned, &pkey, raster ? (size_t)n * Rmax : 1));
     CK(ctx, dmalloc(owned, &pcand, raster ? (size_t)n * Rmax * kPixCand : 1));
+    CK(ctx, dmalloc(owned, &pover, raster ? (size_t)n * kOverWords : 1));
     CK(ctx, dmalloc(owned, &blist, raster ? bcap : 1));
     CK(ctx, dmalloc(owned, &btlist, raster ? bcap : 1));
     CK(ctx, dmalloc(owned, &bcount, 2));
@@ -2417,6 +2425,7 @@ srp_status srp_propagate_batch(srp_ctx *ctx, const srp_prop_params *p, int32_t n
             a.rast_tris = max_tris;
             a.pix_key = pkey;
             a.pix_cand = pcand;
+            a.pix_over = pover;
             a.big = blist;
             a.big_cap = (int)bcap;
             a.big_count = bcount;
@@ -2430,6 +2439,8 @@ srp_status srp_propagate_batch(srp_ctx *ctx, const srp_prop_params *p, int32_t n
                 a.qstate = qst;
             }
         }
+        if (few_trace(na, Rmax, ms, raster, max_tris) && !queue)
+            for (int k = 0; k < na; k++) a.few_tiles += dd[k].tiles;
         cudaGraph_t graph = nullptr;
         CK(ctx, cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
         cudaError_t e = cudaSuccess;

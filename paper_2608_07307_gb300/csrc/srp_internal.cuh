@@ -143,6 +143,7 @@ struct MeshDev {
     int n_static_tris, n_static_nodes, n_static_verts;
     int n_dyn_tris, n_dyn_nodes, n_dyn_verts;
     int max_depth;
+    int stack_need;             // traversal stack entries of the deepest part's 4-wide tree (<= kStack)
     double pad;                 // absolute AABB padding (m)
     double R;                   // bound on |x| over all poses (m)
     double c_ref[3];
@@ -234,6 +235,7 @@ struct TraceArgs {
     unsigned long long *pix_key; // [S][ray_stride] nearest certain FP32 hit: t bits << 32 | 7 - (uncertain
                                  // triangles, at most kPixCand + 1) << 29 | part << 24 | tl; ~0 none
     unsigned *pix_cand;          // [S][ray_stride][kPixCand] the first kPixCand uncertain triangles
+    unsigned *pix_over;          // [S][kOverWords] further uncertain triangles of the slot's pixels (slot_over)
     int4 *big;                   // [big_cap] (slot, sorted triangle, chunk column, chunk row): chunks of large
                                  // triangles that can meet them
     unsigned *big_count;         // entries claimed in big (reset by k_frame)
@@ -249,6 +251,7 @@ struct TraceArgs {
     int *dcnt;                   // [S][ray_stride] emissions of each primary ray, then their exclusive prefix
     int *dtot;                   // [S] emissions of the slot
     int walk_limit_test;         // 1: every BVH walk is bounded at one step (tests of the bound's error path)
+    int few_tiles;               // > 0: the slots' tiles in all, traced by k_trace_few (few_trace)
     int sum_mode;                // sums above the tile: 0 FP64, 1 compensated FP32, 2 plain FP32
     int ctx_parts, hpt_segs;     // most parts / segments over the launch's slots (the trace kernels' shared memory; 0: the maxima)
     // work queue (queue != 0): the raster's second pass and the trace as one
@@ -262,6 +265,27 @@ struct TraceArgs {
 constexpr int kQHead = 0, kQAbort = 1, kQSlot = 2;  // qstate layout; 3 words per slot from kQSlot
 constexpr int kQueueBlocksPerSM = 8;
 inline size_t qstate_words(size_t slots) { return (size_t)kQSlot + 3 * slots; }
+// Launch shapes by batch: a launch of few slots (a propagation stage) is
+// latency-bound, so the frame kernel clears the pixel keys, the second raster
+// pass is one launch and the trace spreads each tile over a block; with many
+// slots the launches overlap other lanes' traces, where separate launches and a
+// warp a tile measured faster.
+constexpr int kFewSlots = 4;
+inline bool few_slots(int S) { return S < kFewSlots; }
+// Does k_trace_few trace the launch?  It wins where the launch waits for its
+// slowest warps, that is for few rays and long walks: the one-lane kernel's time
+// on one evaluation is 45, 58, 90, 130, 180 us of tail at 900, 3k, 12k, 50k and
+// 200k triangles (plus its throughput time), k_trace_few's 28 us plus 0.18 us per
+// 1000 rays.  Measured on single evaluations (old / few, us): 900 triangles 256^2
+// 45 / 41, 512^2 51 / 67; 3k 256^2 58 / 42, 512^2 66 / 65; 12k 512^2 90 / 70; 50k
+// 512^2 130 / 75, 777^2 (2 bounces) 224 / 146, 1024^2 157 / 162; 200k 256^2 148 /
+// 60, 512^2 184 / 87, 1024^2 (2 bounces) 332 / 219, 1448^2 284 / 318: the line
+// rays = 4000 sqrt(triangles) lies between the two everywhere.
+inline bool few_trace(int S, size_t rays, int nseg, bool raster, int n_tris)
+{
+    const double r = (double)S * (double)rays;
+    return few_slots(S) && nseg > 1 && raster && r * r <= 1.6e7 * (double)n_tris;
+}
 constexpr int kDiffBlocks = 64;  // k_diffuse blocks per slot (fixed: the sums have a fixed order)
 // One hit that emits diffuse secondary rays: the FP64 point and lit-side
 // normal from the replay of its ray's specular chain, the weight of one sample
@@ -271,7 +295,10 @@ struct DEmit {
     int src, pad_;
     unsigned long long c0;
 };
-constexpr int kPixCand = 2;      // uncertain triangles kept per pixel (more: the ray traverses)
+constexpr int kPixCand = 2;      // uncertain triangles kept per pixel; up to kPixMax with the slot's list of
+constexpr int kPixMax = 6;       // further ones (more: the ray traverses)
+constexpr int kOverCap = 511;    // entries of that list
+constexpr int kOverWords = 2 * (kOverCap + 1);
 constexpr int kRastSmall = 64;   // largest pixel box one thread rasterises
 constexpr int kRastChunk = 16;   // larger triangles: chunks of 16 x 16 pixels, one warp each
 constexpr int kRastBigBlocksPerSM = 2;  // k_raster_big grid: blocks of 8 warps per SM and 8 slots, one listed chunk a warp
