@@ -9,11 +9,17 @@
 // trajectory, k_prop_accel forms the stage derivative; k_prop_control then
 // accepts or rejects the step and picks the next step size.  All state lives
 // on the device; the host only relaunches the graph and polls a done counter.
-// k_prop_stage runs a warp per trajectory: at the first stage of a step, lanes
-// compute the Sun positions of all stages (their times are fixed with the step
-// size), lanes 0-5 form the stage state.  Without ray tracing between the
-// stages (a SPAD table, read by spad_lookup in the acceleration, or SRP off)
-// the whole step is one kernel, k_prop_step, built from the same parts.
+// Every kernel of a step runs a warp per trajectory on a copy of its state in
+// shared memory.  An FP64 instruction holds this GPU's FP64 pipe for 64 cycles a
+// warp whatever the number of active lanes (a dependent chain and four independent
+// ones measured the same; a square root or a division takes 10 of them, atan2 45,
+// pow 92), so what these kernels cost is the number of FP64 instructions their warp
+// issues: components, norms and divisions are spread over the lanes, and one
+// instruction serves all of them.  Each value is formed by the expression a single
+// lane would use.  At the first stage of a step, lanes compute the Sun positions of
+// all stages (their times are fixed with the step size).  Without ray tracing between
+// the stages (a SPAD table or SRP off) the whole step is one kernel, k_prop_step,
+// built from the same parts.
 //
 // Integrators: Fehlberg's 7(8) pair (13 stages, NASA TR R-287, 1968),
 // propagating the 7th-order solution, error norm
@@ -98,44 +104,6 @@ __device__ void lvlh_matrix(const double *y, double *L)
     for (int k = 0; k < 3; k++) { L[3 * k] = xb[k]; L[3 * k + 1] = yb[k]; L[3 * k + 2] = zb[k]; }
 }
 
-// body -> inertial rotation, row-major: Q (inertial attitude) or LVLH(y) Q
-// (the LVLH frame turned by the constant quaternion whose rotation is Q)
-__device__ void body_to_inertial(int attitude, const double *Q, const double *y, double *R)
-{
-    if (attitude == 1) {
-        for (int k = 0; k < 9; k++) R[k] = Q[k];
-        return;
-    }
-    double L[9];
-    lvlh_matrix(y, L);
-    for (int i = 0; i < 3; i++)
-        for (int j = 0; j < 3; j++) R[3 * i + j] = L[3 * i] * Q[j] + L[3 * i + 1] * Q[3 + j] + L[3 * i + 2] * Q[6 + j];
-}
-
-// Gravity of the configured bodies at (t, y).
-__device__ void gravity(const PropDev &P, int central, const double *y, const double *rs, double *a)
-{
-    double r2 = y[0] * y[0] + y[1] * y[1] + y[2] * y[2], r = sqrt(r2);
-    double mu = central == 1 ? kMuSun : kMuEarth;
-    const double ir3 = 1.0 / (r2 * r);
-    for (int k = 0; k < 3; k++) a[k] = -mu * y[k] * ir3;
-    if (central == 0 && P.j2) {
-        const double ir2 = 1.0 / r2;
-        double z2 = y[2] * y[2] * ir2;
-        double f = -1.5 * kJ2 * kMuEarth * kREarth * kREarth * (ir3 * ir2);
-        a[0] += f * y[0] * (1.0 - 5.0 * z2);
-        a[1] += f * y[1] * (1.0 - 5.0 * z2);
-        a[2] += f * y[2] * (3.0 - 5.0 * z2);
-    }
-    if (central == 0 && P.sun3) {
-        double d[3] = {rs[0] - y[0], rs[1] - y[1], rs[2] - y[2]};
-        double dn = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-        double sn = sqrt(rs[0] * rs[0] + rs[1] * rs[1] + rs[2] * rs[2]);
-        const double id3 = 1.0 / (dn * dn * dn), is3 = 1.0 / (sn * sn * sn);
-        for (int k = 0; k < 3; k++) a[k] += kMuSun * (d[k] * id3 - rs[k] * is3);
-    }
-}
-
 // cfg (null: P's values for every trajectory): [n][8] central, attitude, q[4], mass, unused
 __global__ void k_prop_init(PropState *S, int n, const double *y0, const double *t01, PropDev P, const double *cfg,
                             int *n_done)
@@ -156,6 +124,7 @@ __global__ void k_prop_init(PropState *S, int n, const double *y0, const double 
         for (int k = 0; k < 4; k++) X.q[k] = P.q[k];
         X.mass = P.mass;
     }
+    X.imass = 1.0 / X.mass;
     quat_matrix(X.q, X.Qm);
     for (int k = 0; k < 6; k++) X.y[k] = y0[6 * i + k];
     X.t = t01[2 * i];
@@ -172,45 +141,48 @@ __global__ void k_prop_init(PropState *S, int n, const double *y0, const double 
     if (X.done) atomicAdd(n_done, 1);
 }
 
-// Lane 0's part of a stage: time, Sun direction in the body frame and
-// distance (negative to skip the SRP call), shadow, attitude.
-__device__ __forceinline__ void stage_tail(PropState &X, int i, const PropDev &P, int stage, double *sun_dir,
-                                           double *sun_dist)
+// Warps (trajectories) of a block: one to each of an SM's four FP64 pipes.
+constexpr int kPropWarps = 4;
+
+// A trajectory's warp: its state, and the operands that lanes hand to each other.
+struct PropWarp {
+    PropState X;
+    double y[6], h[3], sv[3], rs[3];  // stage state, r x v, Sun from spacecraft, Sun (stage_body)
+    double q[11];                     // the stage's quotients
+    double zb[3], yb[3], xb[3], e[3]; // LVLH axes, Sun direction from the central body
+    double sun[3], dist;              // body-frame Sun direction and distance (AU; negative: no SRP)
+};
+
+// The state's words in and out of shared memory: independent loads, one latency.
+__device__ __forceinline__ void load_state(PropWarp &W, const PropState &G, int lane)
 {
-    const int rk4 = P.method == 1;
-    X.ts = X.t + (rk4 ? cC4[stage] : cC[stage]) * X.hs;
-    // Sun direction and distance
-    double rs[3] = {0.0, 0.0, 0.0}, sv[3];
-    if (X.central == 0)
-        for (int k = 0; k < 3; k++) rs[k] = X.rs_st[stage][k];
-    for (int k = 0; k < 3; k++) { X.rsun[k] = rs[k]; sv[k] = rs[k] - X.ys[k]; }
-    double sd = sqrt(sv[0] * sv[0] + sv[1] * sv[1] + sv[2] * sv[2]);
-    for (int k = 0; k < 3; k++) sv[k] /= sd;
-    // cylindrical Earth shadow
-    X.shadow = 0;
-    if (X.central == 0) {
-        const double irsn = 1.0 / sqrt(rs[0] * rs[0] + rs[1] * rs[1] + rs[2] * rs[2]);
-        double e[3] = {rs[0] * irsn, rs[1] * irsn, rs[2] * irsn};
-        double pr = X.ys[0] * e[0] + X.ys[1] * e[1] + X.ys[2] * e[2];
-        double q[3] = {X.ys[0] - pr * e[0], X.ys[1] - pr * e[1], X.ys[2] - pr * e[2]};
-        if (pr < 0.0 && q[0] * q[0] + q[1] * q[1] + q[2] * q[2] < kREarth * kREarth) X.shadow = 1;
-    }
-    double R[9];
-    body_to_inertial(X.attitude, X.Qm, X.ys, R);
-    for (int k = 0; k < 9; k++) X.R[k] = R[k];
-    for (int k = 0; k < 3; k++) sun_dir[3 * i + k] = R[k] * sv[0] + R[3 + k] * sv[1] + R[6 + k] * sv[2];
-    // finished and shadowed trajectories skip their SRP evaluation (negative distance)
-    sun_dist[i] = (X.done || X.shadow || !P.srp) ? -1.0 : sd / kAU;
+    static_assert(sizeof(PropState) % 8 == 0, "copied by 8-byte words");
+    const double *src = reinterpret_cast<const double *>(&G);
+    double *dst = reinterpret_cast<double *>(&W.X);
+#pragma unroll
+    for (int k = 0; k < (int)(sizeof(PropState) / 8); k += 32)
+        if (k + lane < (int)(sizeof(PropState) / 8)) dst[k + lane] = src[k + lane];
+    __syncwarp();
+}
+__device__ __forceinline__ void store_state(const PropWarp &W, PropState &G, int lane)
+{
+    __syncwarp();
+    const double *src = reinterpret_cast<const double *>(&W.X);
+    double *dst = reinterpret_cast<double *>(&G);
+#pragma unroll
+    for (int k = 0; k < (int)(sizeof(PropState) / 8); k += 32)
+        if (k + lane < (int)(sizeof(PropState) / 8)) dst[k + lane] = src[k + lane];
 }
 
-// Stage state, Sun direction (body frame) and distance for the SRP call; a
-// warp per trajectory.  At the first stage of a step, once the step size is
-// fixed, every stage time is known: lanes compute the Sun positions of all
-// stages at once.  Lanes 0-5 form the six components of the stage state; lane
-// 0 the rest.
-__device__ __forceinline__ void stage_body(PropState &X, int i, const PropDev &P, int stage, int lane, double *sun_dir,
-                                           double *sun_dist)
+__device__ __forceinline__ double shfl(double x, int lane) { return __shfl_sync(0xffffffffu, x, lane); }
+
+// Stage state, gravity, attitude, Sun direction (body frame) and distance for
+// the SRP call (negative to skip it: a finished or shadowed trajectory).  At the
+// first stage of a step, once the step size is fixed, every stage time is known:
+// lanes compute the Sun positions of all stages at once.
+__device__ __forceinline__ void stage_body(PropWarp &W, int i, const PropDev &P, int stage, int lane)
 {
+    PropState &X = W.X;
     const int rk4 = P.method == 1;
     if (stage == 0) {
         if (lane == 0 && !X.done) {
@@ -229,173 +201,344 @@ __device__ __forceinline__ void stage_body(PropState &X, int i, const PropDev &P
             sun_pos(P.epoch_mjd_tt + ts / 86400.0, rs);
             for (int k = 0; k < 3; k++) X.rs_st[lane][k] = rs[k];
         }
+        __syncwarp();
     }
-    if (lane < 6) {
-        const int k = lane;
-        double acc = 0.0;
+    const int c3 = lane % 3;
+    // lanes 0-5: the components of the stage state; lane 6: the stage time
+    {
+        double acc = 0.0, base = X.t;
+        if (lane < 6) base = X.y[lane];
+        if (lane == 6) acc = rk4 ? cC4[stage] : cC[stage];
+        const int k = lane < 6 ? lane : 0;
         if (rk4) {
-            if (stage > 0) acc = 0.5 * X.k[stage - 1][k] * (stage == 3 ? 2.0 : 1.0);
+            if (stage > 0) {
+                const double x = 0.5 * X.k[stage - 1][k] * (stage == 3 ? 2.0 : 1.0);
+                if (lane < 6) acc = x;
+            }
         } else {
-            for (int j = 0; j < stage; j++) acc += cA[stage][j] * X.k[j][k];
+            double s = 0.0;
+            for (int j = 0; j < stage; j++) s += cA[stage][j] * X.k[j][k];
+            if (lane < 6) acc = s;
         }
-        X.ys[k] = X.y[k] + X.hs * acc;
+        const double x = base + X.hs * acc;
+        if (lane < 6) W.y[lane] = X.ys[lane] = x;
+        if (lane == 6) X.ts = x;
+        if (lane < 3) W.rs[lane] = X.central == 0 ? X.rs_st[stage][lane] : 0.0;
     }
     __syncwarp();
-    if (lane != 0) return;
-    stage_tail(X, i, P, stage, sun_dir, sun_dist);
-}
-
-__global__ void k_prop_stage(PropState *S, int n, PropDev P, int stage, double *sun_dir, double *sun_dist)
-{
-    pdl_enter();
-    const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (i >= n) return;  // whole warps (blocks are multiples of 32 threads)
-    stage_body(S[i], i, P, stage, threadIdx.x & 31, sun_dir, sun_dist);
-}
-
-// Stage derivative: gravity plus the SRP force (traced, or the SPAD interpolant).
-__device__ __forceinline__ void accel_body(PropState &X, int i, const PropDev &P, int stage, const double *force,
-                                           const double *sun_dir, const double *sun_dist)
-{
-    double a[3];
-    gravity(P, X.central, X.ys, X.rsun, a);
-    if (P.srp && !X.shadow) {
-        double Fs[6];
-        const double *F = force + 3 * i;
-        if (P.spad.table) {
-            // SPAD interpolation (Sec. 4.2) at this stage's body-frame Sun direction
-            spad_lookup(P.spad, sun_dir + 3 * i, sun_dist[i], Fs);
-            F = Fs;
-        }
-        const double im = 1.0 / X.mass;
-        for (int k = 0; k < 3; k++) a[k] += (X.R[3 * k] * F[0] + X.R[3 * k + 1] * F[1] + X.R[3 * k + 2] * F[2]) * im;
+    // lanes 0-2: r x v; the others: the Sun from the spacecraft (a product with one is exact)
+    {
+        const int k1 = c3 == 2 ? 0 : c3 + 1, k2 = c3 == 0 ? 2 : c3 - 1;
+        const bool hv = lane < 3;
+        const double p = hv ? W.y[k1] : W.rs[c3], q = hv ? W.y[3 + k2] : 1.0;
+        const double r = hv ? W.y[k2] : W.y[c3], s = hv ? W.y[3 + k1] : 1.0;
+        const double x = p * q - r * s;
+        if (lane < 3) W.h[lane] = x;
+        else if (lane < 6) W.sv[c3] = x;
     }
-    for (int k = 0; k < 3; k++) { X.k[stage][k] = X.ys[3 + k]; X.k[stage][3 + k] = a[k]; }
-    if (!X.done) X.evals++;
+    __syncwarp();
+    // norms: lane 0 |r|, 1 |r x v|, 2 Sun distance, 3 |Sun|
+    double n2, n;
+    {
+        const int g = lane & 3;
+        const double *v = g == 0 ? W.y : g == 1 ? W.h : g == 2 ? W.sv : W.rs;
+        n2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
+        n = sqrt(n2);
+    }
+    const double r2 = shfl(n2, 0), r = shfl(n, 0), hn = shfl(n, 1), sd = shfl(n, 2), sn = shfl(n, 3);
+    // every quotient of the stage in one division
+    {
+        const double m = lane == 9 ? sn : lane == 8 ? sd : r2;           // cubes: r2 r, |d|^3, |s|^3
+        const double m2 = m * (lane == 9 ? sn : lane == 8 ? sd : r);
+        const double m3 = m2 * (lane == 9 ? sn : sd);
+        double num = 1.0, den = 1.0;
+        const bool lvlh = X.attitude != 1, earth = X.central == 0;
+        if (lane < 3) { num = W.sv[lane]; den = sd; }
+        else if (lane == 3) { num = -1.0; den = lvlh ? r : 1.0; }
+        else if (lane == 4) { num = -1.0; den = lvlh ? hn : 1.0; }
+        else if (lane == 5) den = earth ? sn : 1.0;
+        else if (lane == 6) den = m2;
+        else if (lane == 7) den = r2;
+        else if (lane == 8 || lane == 9) den = earth ? m3 : 1.0;
+        else if (lane == 10) { num = sd; den = kAU; }
+        const double x = num / den;
+        if (lane < 11) W.q[lane] = x;
+    }
+    __syncwarp();
+    // z_b = nadir, y_b = -orbit normal, e = Sun direction from the central body
+    {
+        const int g = lane / 3;
+        const double x = (g == 0 ? W.y[c3] : g == 1 ? W.h[c3] : W.rs[c3]) * W.q[g == 0 ? 3 : g == 1 ? 4 : 5];
+        if (lane < 9) (g == 0 ? W.zb : g == 1 ? W.yb : W.e)[c3] = x;
+    }
+    __syncwarp();
+    // x_b = y_b x z_b, in lanes 0-2
+    {
+        const int k1 = c3 == 2 ? 0 : c3 + 1, k2 = c3 == 0 ? 2 : c3 - 1;
+        const double x = W.yb[k1] * W.zb[k2] - W.yb[k2] * W.zb[k1];
+        if (lane < 3) W.xb[lane] = x;
+    }
+    __syncwarp();
+    // body -> inertial rotation, an element a lane: the quaternion's (inertial attitude) or
+    // the LVLH frame (columns x_b, y_b, z_b) turned by it
+    {
+        const int l = lane < 9 ? lane : 0, a = l / 3, b = l % 3;
+        const double x = W.xb[a] * X.Qm[b] + W.yb[a] * X.Qm[3 + b] + W.zb[a] * X.Qm[6 + b];
+        if (lane < 9) X.R[lane] = X.attitude == 1 ? X.Qm[lane] : x;
+    }
+    // cylindrical Earth shadow
+    int shadow = 0;
+    if (X.central == 0) {
+        const double pr = W.y[0] * W.e[0] + W.y[1] * W.e[1] + W.y[2] * W.e[2];
+        const double q = W.y[c3] - pr * W.e[c3];
+        const double q0 = shfl(q, 0), q1 = shfl(q, 1), q2 = shfl(q, 2);
+        if (pr < 0.0 && q0 * q0 + q1 * q1 + q2 * q2 < kREarth * kREarth) shadow = 1;
+    }
+    // gravity, a component a lane: central body, Earth J2, the Sun as a third body
+    {
+        const double mu = X.central == 1 ? kMuSun : kMuEarth;
+        const double ir3 = W.q[6], yk = W.y[c3];
+        double a = -mu * yk * ir3;
+        if (X.central == 0 && P.j2) {
+            const double ir2 = W.q[7];
+            const double z2 = W.y[2] * W.y[2] * ir2;
+            const double f = -1.5 * kJ2 * kMuEarth * kREarth * kREarth * (ir3 * ir2);
+            a += f * yk * ((c3 == 2 ? 3.0 : 1.0) - 5.0 * z2);
+        }
+        if (X.central == 0 && P.sun3) a += kMuSun * (W.sv[c3] * W.q[8] - W.rs[c3] * W.q[9]);
+        if (lane < 3) X.grav[lane] = a;
+    }
+    __syncwarp();
+    const double dir = X.R[c3] * W.q[0] + X.R[3 + c3] * W.q[1] + X.R[6 + c3] * W.q[2];
+    if (lane < 3) {
+        X.rsun[lane] = W.rs[lane];
+        W.sun[lane] = dir;
+    }
+    if (lane == 0) {
+        X.shadow = shadow;
+        W.dist = (X.done || shadow || !P.srp) ? -1.0 : W.q[10];
+    }
+    __syncwarp();
 }
 
-__global__ void k_prop_accel(PropState *S, int n, PropDev P, int stage, const double *force, const double *sun_dir,
-                             const double *sun_dist)
+// The stage's Sun direction and distance where the SRP call reads them.
+__device__ __forceinline__ void store_sun(const PropWarp &W, int i, int lane, double *sun_dir, double *sun_dist)
+{
+    if (lane < 3) sun_dir[3 * i + lane] = W.sun[lane];
+    if (lane == 3) sun_dist[i] = W.dist;
+}
+
+// What the acceleration of a stage reads of the SRP call: the traced force, or
+// the Sun direction and distance a SPAD table is read at.
+__device__ __forceinline__ void load_srp(PropWarp &W, int i, const PropDev &P, int lane, const double *force,
+                                         const double *sun_dir, const double *sun_dist)
+{
+    if (!P.srp) return;
+    if (P.spad.table) {
+        if (lane < 3) W.sun[lane] = sun_dir[3 * i + lane];
+        if (lane == 3) W.dist = sun_dist[i];
+    } else if (lane < 3) {
+        W.h[lane] = force[3 * i + lane];
+    }
+    __syncwarp();
+}
+
+__global__ void __launch_bounds__(32 * kPropWarps) k_prop_stage(PropState *S, int n, PropDev P, int stage,
+                                                                double *sun_dir, double *sun_dist)
 {
     pdl_enter();
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    accel_body(S[i], i, P, stage, force, sun_dir, sun_dist);
+    __shared__ PropWarp sh[kPropWarps];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int i = blockIdx.x * kPropWarps + w;
+    if (i >= n) return;  // whole warps
+    PropWarp &W = sh[w];
+    load_state(W, S[i], lane);
+    stage_body(W, i, P, stage, lane);
+    store_sun(W, i, lane, sun_dir, sun_dist);
+    store_state(W, S[i], lane);
 }
 
-// Step control: accept or reject, next step size, completion.
-__device__ __forceinline__ void control_body(PropState &X, int i, const PropDev &P, int *n_done, double *h_log,
+// spad_lookup's force by a warp, component `lane` in lanes 0-2: both angles in one
+// atan2, the quotients in one division.
+__device__ __forceinline__ double spad_force_warp(const SpadDev &g, const double *s, double dist, int lane)
+{
+    if (dist < 0.0) return 0.0;
+    const bool elev = lane == 1;
+    const double hyp = hypot(s[0], s[1]);
+    const double a = atan2(elev ? s[2] : s[1], elev ? hyp : s[0]) - (elev ? g.el0 : g.az0);
+    const double u = a * (g.n_az * 0.15915494309189535);  // cells of 2 pi / n_az
+    const double q = (lane == 2 ? 1.0 : elev ? a : u) / (lane == 2 ? dist * dist : elev ? g.d_el : (double)g.n_az);
+    const SpadCell c = spad_cell(g, shfl(u, 0), shfl(q, 0), shfl(q, 1));
+    return spad_value(c, lane % 3, shfl(q, 2));
+}
+
+// Stage derivative: gravity plus the SRP force (traced, in W.h, or the SPAD
+// interpolant, Sec. 4.2, at this stage's body-frame Sun direction).
+__device__ __forceinline__ void accel_body(PropWarp &W, const PropDev &P, int stage, int lane)
+{
+    PropState &X = W.X;
+    const int c3 = lane % 3;
+    double a = X.grav[c3];
+    if (P.srp && !X.shadow) {
+        if (P.spad.table) {
+            const double f = spad_force_warp(P.spad, W.sun, W.dist, lane);
+            if (lane < 3) W.h[lane] = f;
+            __syncwarp();
+        }
+        a += (X.R[3 * c3] * W.h[0] + X.R[3 * c3 + 1] * W.h[1] + X.R[3 * c3 + 2] * W.h[2]) * X.imass;
+    }
+    if (lane < 3) X.k[stage][lane] = X.ys[3 + lane];
+    else if (lane < 6) X.k[stage][lane] = a;
+    if (lane == 0 && !X.done) X.evals++;
+    __syncwarp();
+}
+
+__global__ void __launch_bounds__(32 * kPropWarps) k_prop_accel(PropState *S, int n, PropDev P, int stage,
+                                                                const double *force, const double *sun_dir,
+                                                                const double *sun_dist)
+{
+    pdl_enter();
+    __shared__ PropWarp sh[kPropWarps];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int i = blockIdx.x * kPropWarps + w;
+    if (i >= n) return;  // whole warps
+    PropWarp &W = sh[w];
+    load_srp(W, i, P, lane, force, sun_dir, sun_dist);
+    load_state(W, S[i], lane);
+    accel_body(W, P, stage, lane);
+    store_state(W, S[i], lane);
+}
+
+// Step control: accept or reject, next step size, completion.  Lanes 0-5 hold a
+// component of the state each; lane 0 decides.
+__device__ __forceinline__ void control_body(PropWarp &W, int i, const PropDev &P, int lane, int *n_done, double *h_log,
                                              int64_t h_cap)
 {
-    if (X.done) return;
+    PropState &X = W.X;
+    if (X.done) return;  // uniform
     const double h = X.hs;
+    const int k = lane < 6 ? lane : 0;
     if (P.n_replay > 0) {
         // replay: take the given step, 7th-order solution, no error control
-        for (int k = 0; k < 6; k++) {
-            double s7 = 0.0;
-            for (int j = 0; j < 13; j++) s7 += cB7[j] * X.k[j][k];
-            X.y[k] = X.y[k] + h * s7;
+        double s7 = 0.0;
+        for (int j = 0; j < 13; j++) s7 += cB7[j] * X.k[j][k];
+        const double yn = X.y[k] + h * s7;
+        __syncwarp();
+        if (lane < 6) X.y[k] = yn;
+        if (lane == 0) {
+            X.t += h;
+            if (h_log && X.nlog < h_cap) h_log[(size_t)i * h_cap + X.nlog] = h;
+            X.nlog++;
+            X.steps++;
+            if (X.steps >= P.n_replay) { X.done = 1; atomicAdd(n_done, 1); }
         }
-        X.t += h;
-        if (h_log && X.nlog < h_cap) h_log[(size_t)i * h_cap + X.nlog] = h;
-        X.nlog++;
-        X.steps++;
-        if (X.steps >= P.n_replay) { X.done = 1; atomicAdd(n_done, 1); }
+        __syncwarp();
         return;
     }
     const bool last = X.t + X.h >= X.t1;
     bool accept = true;
-    double yn[6];
+    double yn;
     double fac = 1.0;
     if (P.method == 1) {
-        for (int k = 0; k < 6; k++) {
-            double acc = 0.0;
-            for (int j = 0; j < 4; j++) acc += cB4[j] * X.k[j][k];
-            yn[k] = X.y[k] + h * acc;
-        }
+        double acc = 0.0;
+        for (int j = 0; j < 4; j++) acc += cB4[j] * X.k[j][k];
+        yn = X.y[k] + h * acc;
     } else {
+        double s7 = 0.0, s8 = 0.0;
+        for (int j = 0; j < 13; j++) { s7 += cB7[j] * X.k[j][k]; s8 += cB8[j] * X.k[j][k]; }
+        yn = X.y[k] + h * s7;
+        const double sc = (k < 3 ? P.atol_pos : P.atol_vel) + P.rtol * fmax(fabs(X.y[k]), fabs(yn));
+        const double ek = fabs(h * (s7 - s8)) / sc;
         double e = 0.0;
-        for (int k = 0; k < 6; k++) {
-            double s7 = 0.0, s8 = 0.0;
-            for (int j = 0; j < 13; j++) { s7 += cB7[j] * X.k[j][k]; s8 += cB8[j] * X.k[j][k]; }
-            yn[k] = X.y[k] + h * s7;
-            double sc = (k < 3 ? P.atol_pos : P.atol_vel) + P.rtol * fmax(fabs(X.y[k]), fabs(yn[k]));
-            e = fmax(e, fabs(h * (s7 - s8)) / sc);
-        }
+        for (int j = 0; j < 6; j++) e = fmax(e, shfl(ek, j));
         fac = e == 0.0 ? 5.0 : fmin(5.0, fmax(0.2, 0.9 * pow(e, -1.0 / 8.0)));
         accept = e <= 1.0;
     }
-    if (accept) {
-        for (int k = 0; k < 6; k++) X.y[k] = yn[k];
-        // fixed steps snap onto t1 when they land within 1e-9 of a step of it
-        X.t = (last || (P.method == 1 && X.t1 - (X.t + h) < 1e-9 * P.h0)) ? X.t1 : X.t + h;
-        if (h_log && X.nlog < h_cap) h_log[(size_t)i * h_cap + X.nlog] = h;
-        X.nlog++;
-        X.steps++;
-    } else {
-        X.rejects++;
+    __syncwarp();
+    if (accept && lane < 6) X.y[k] = yn;
+    if (lane == 0) {
+        if (accept) {
+            // fixed steps snap onto t1 when they land within 1e-9 of a step of it
+            X.t = (last || (P.method == 1 && X.t1 - (X.t + h) < 1e-9 * P.h0)) ? X.t1 : X.t + h;
+            if (h_log && X.nlog < h_cap) h_log[(size_t)i * h_cap + X.nlog] = h;
+            X.nlog++;
+            X.steps++;
+        } else {
+            X.rejects++;
+        }
+        if (P.method == 0) {
+            double hn = X.hs * fac;
+            if (P.h_max > 0.0) hn = fmin(hn, P.h_max);
+            if (X.t < X.t1 && hn < P.h_min) { X.status = SRP_ERR_STEP; X.done = 1; }
+            X.h = hn;
+        }
+        if (X.t >= X.t1) X.done = 1;
+        if (X.steps + X.rejects > P.max_steps && !X.done) { X.status = SRP_ERR_STEP; X.done = 1; }
+        if (X.done) atomicAdd(n_done, 1);
     }
-    if (P.method == 0) {
-        double hn = X.hs * fac;
-        if (P.h_max > 0.0) hn = fmin(hn, P.h_max);
-        if (X.t < X.t1 && hn < P.h_min) { X.status = SRP_ERR_STEP; X.done = 1; }
-        X.h = hn;
-    }
-    if (X.t >= X.t1) X.done = 1;
-    if (X.steps + X.rejects > P.max_steps && !X.done) { X.status = SRP_ERR_STEP; X.done = 1; }
-    if (X.done) atomicAdd(n_done, 1);
+    __syncwarp();
 }
 
-__global__ void k_prop_control(PropState *S, int n, PropDev P, int *n_done, double *h_log, int64_t h_cap)
+__global__ void __launch_bounds__(32 * kPropWarps) k_prop_control(PropState *S, int n, PropDev P, int *n_done,
+                                                                  double *h_log, int64_t h_cap)
 {
     pdl_enter();
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    control_body(S[i], i, P, n_done, h_log, h_cap);
+    __shared__ PropWarp sh[kPropWarps];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int i = blockIdx.x * kPropWarps + w;
+    if (i >= n) return;  // whole warps
+    PropWarp &W = sh[w];
+    load_state(W, S[i], lane);
+    control_body(W, i, P, lane, n_done, h_log, h_cap);
+    store_state(W, S[i], lane);
 }
 
 // The stage derivative of `stage` and, in the same launch, the state of the
 // next stage; after the last stage, step control and the first stage of the
-// next step (which the captured step then starts from).  A warp per trajectory.
-__global__ void k_prop_next(PropState *S, int n, PropDev P, int stage, const double *force, double *sun_dir,
-                            double *sun_dist, int *n_done, double *h_log, int64_t h_cap)
+// next step (which the captured step then starts from).
+__global__ void __launch_bounds__(32 * kPropWarps) k_prop_next(PropState *S, int n, PropDev P, int stage,
+                                                               const double *force, double *sun_dir, double *sun_dist,
+                                                               int *n_done, double *h_log, int64_t h_cap)
 {
     pdl_enter();
-    const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
+    __shared__ PropWarp sh[kPropWarps];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int i = blockIdx.x * kPropWarps + w;
     if (i >= n) return;  // whole warps
-    PropState &X = S[i];
+    PropWarp &W = sh[w];
     const int nst = P.method == 1 ? 4 : 13;
-    if (lane == 0) accel_body(X, i, P, stage, force, sun_dir, sun_dist);
-    __syncwarp();
-    if (stage + 1 < nst) {
-        stage_body(X, i, P, stage + 1, lane, sun_dir, sun_dist);
-        return;
-    }
-    if (lane == 0) control_body(X, i, P, n_done, h_log, h_cap);
-    __syncwarp();
-    stage_body(X, i, P, 0, lane, sun_dir, sun_dist);
+    load_srp(W, i, P, lane, force, sun_dir, sun_dist);
+    load_state(W, S[i], lane);
+    accel_body(W, P, stage, lane);
+    const bool end = stage + 1 >= nst;
+    if (end) control_body(W, i, P, lane, n_done, h_log, h_cap);
+    stage_body(W, i, P, end ? 0 : stage + 1, lane);
+    store_sun(W, i, lane, sun_dir, sun_dist);
+    store_state(W, S[i], lane);
 }
 
 // A whole step in one launch when no ray-traced evaluation sits between the
 // stages (SPAD table or SRP off): the stage, acceleration and control parts of
-// the kernels above, in their order, a warp per trajectory.
-__global__ void k_prop_step(PropState *S, int n, PropDev P, double *sun_dir, double *sun_dist, int *n_done,
-                            double *h_log, int64_t h_cap)
+// the kernels above, in their order.
+__global__ void __launch_bounds__(32 * kPropWarps) k_prop_step(PropState *S, int n, PropDev P, double *sun_dir,
+                                                               double *sun_dist, int *n_done, double *h_log,
+                                                               int64_t h_cap)
 {
     pdl_enter();
-    const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
+    __shared__ PropWarp sh[kPropWarps];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int i = blockIdx.x * kPropWarps + w;
     if (i >= n) return;  // whole warps
-    PropState &X = S[i];
+    PropWarp &W = sh[w];
+    load_state(W, S[i], lane);
     const int nst = P.method == 1 ? 4 : 13;
     for (int stage = 0; stage < nst; stage++) {
-        stage_body(X, i, P, stage, lane, sun_dir, sun_dist);
-        __syncwarp();
-        if (lane == 0) accel_body(X, i, P, stage, nullptr, sun_dir, sun_dist);
-        __syncwarp();
+        stage_body(W, i, P, stage, lane);
+        accel_body(W, P, stage, lane);
     }
-    if (lane == 0) control_body(X, i, P, n_done, h_log, h_cap);
+    store_sun(W, i, lane, sun_dir, sun_dist);
+    control_body(W, i, P, lane, n_done, h_log, h_cap);
+    store_state(W, S[i], lane);
 }
 
 
@@ -612,28 +755,28 @@ cudaError_t launch_prop_init(PropState *S, int n, const double *y0, const double
 cudaError_t launch_prop_stage(PropState *S, int n, const PropDev &P, int stage, double *sun_dir, double *sun_dist,
                               cudaStream_t st)
 {
-    return launch_chained(k_prop_stage, dim3((n + 3) / 4), dim3(128), 0, st, S, n, P, stage, sun_dir, sun_dist);  // a warp per trajectory
+    return launch_chained(k_prop_stage, dim3((n + kPropWarps - 1) / kPropWarps), dim3(32 * kPropWarps), 0, st, S, n, P, stage, sun_dir, sun_dist);
 }
 cudaError_t launch_prop_accel(PropState *S, int n, const PropDev &P, int stage, const double *force, cudaStream_t st,
                               const double *sun_dir, const double *sun_dist)
 {
-    return launch_chained(k_prop_accel, dim3((n + 63) / 64), dim3(64), 0, st, S, n, P, stage, force, sun_dir, sun_dist);
+    return launch_chained(k_prop_accel, dim3((n + kPropWarps - 1) / kPropWarps), dim3(32 * kPropWarps), 0, st, S, n, P, stage, force, sun_dir, sun_dist);
 }
 cudaError_t launch_prop_next(PropState *S, int n, const PropDev &P, int stage, const double *force, double *sun_dir,
                              double *sun_dist, int *n_done, double *h_log, int64_t h_cap, cudaStream_t st)
 {
-    return launch_chained(k_prop_next, dim3((n + 3) / 4), dim3(128), 0, st, S, n, P, stage, force, sun_dir, sun_dist,
+    return launch_chained(k_prop_next, dim3((n + kPropWarps - 1) / kPropWarps), dim3(32 * kPropWarps), 0, st, S, n, P, stage, force, sun_dir, sun_dist,
                           n_done, h_log, h_cap);
 }
 cudaError_t launch_prop_step(PropState *S, int n, const PropDev &P, double *sun_dir, double *sun_dist, int *n_done,
                              double *h_log, int64_t h_cap, cudaStream_t st)
 {
-    return launch_chained(k_prop_step, dim3((n + 3) / 4), dim3(128), 0, st, S, n, P, sun_dir, sun_dist, n_done, h_log, h_cap);
+    return launch_chained(k_prop_step, dim3((n + kPropWarps - 1) / kPropWarps), dim3(32 * kPropWarps), 0, st, S, n, P, sun_dir, sun_dist, n_done, h_log, h_cap);
 }
 cudaError_t launch_prop_control(PropState *S, int n, const PropDev &P, int *n_done, double *h_log, int64_t h_cap,
                                 cudaStream_t st)
 {
-    return launch_chained(k_prop_control, dim3((n + 63) / 64), dim3(64), 0, st, S, n, P, n_done, h_log, h_cap);
+    return launch_chained(k_prop_control, dim3((n + kPropWarps - 1) / kPropWarps), dim3(32 * kPropWarps), 0, st, S, n, P, n_done, h_log, h_cap);
 }
 
 cudaError_t launch_prop_ckpt(PropState *S, int n, double *buf, bool save, double h0, cudaStream_t st)

@@ -313,23 +313,19 @@ struct SpadDev {
     double az0, el0, d_el;
 };
 
-// Bilinear interpolant of the SPAD table at body-frame direction s and Sun
-// distance dist (AU; negative gives zeros): out = [F, T] scaled by 1/dist^2.
-// Azimuth is periodic over n_az cells; elevation clamps to the outer rows.
-__device__ __forceinline__ void spad_lookup(const SpadDev &g, const double *s, double dist, double out[6])
+// The four samples about a direction and their weights: u in cells of azimuth
+// (periodic over n_az, uq = u / n_az), v in cells of elevation (clamped to the
+// outer rows).
+struct SpadCell {
+    const double *t00, *t01, *t10, *t11;
+    double w00, w01, w10, w11;
+};
+__device__ __forceinline__ SpadCell spad_cell(const SpadDev &g, double u, double uq, double v)
 {
-    if (dist < 0.0) {
-        for (int k = 0; k < 6; k++) out[k] = 0.0;
-        return;
-    }
-    const double az = atan2(s[1], s[0]);
-    const double el = atan2(s[2], hypot(s[0], s[1]));
-    double u = (az - g.az0) * (g.n_az * 0.15915494309189535);  // cells of 2 pi / n_az
-    u -= floor(u / g.n_az) * g.n_az;                          // into [0, n_az]
+    u -= floor(uq) * g.n_az;  // into [0, n_az]
     const int i0 = min((int)u, g.n_az - 1);
     const double fa = u - i0;
     const int i1 = i0 + 1 == g.n_az ? 0 : i0 + 1;
-    const double v = (el - g.el0) / g.d_el;
     int j0 = 0, j1 = 0;
     double fe = 0.0;
     if (g.n_el > 1 && v > 0.0) {
@@ -341,12 +337,36 @@ __device__ __forceinline__ void spad_lookup(const SpadDev &g, const double *s, d
             fe = v - j0;
         }
     }
-    const double w00 = (1.0 - fa) * (1.0 - fe), w01 = fa * (1.0 - fe), w10 = (1.0 - fa) * fe, w11 = fa * fe;
-    const double *t00 = g.table + 6 * ((size_t)j0 * g.n_az + i0), *t01 = g.table + 6 * ((size_t)j0 * g.n_az + i1);
-    const double *t10 = g.table + 6 * ((size_t)j1 * g.n_az + i0), *t11 = g.table + 6 * ((size_t)j1 * g.n_az + i1);
+    SpadCell c;
+    c.w00 = (1.0 - fa) * (1.0 - fe);
+    c.w01 = fa * (1.0 - fe);
+    c.w10 = (1.0 - fa) * fe;
+    c.w11 = fa * fe;
+    c.t00 = g.table + 6 * ((size_t)j0 * g.n_az + i0);
+    c.t01 = g.table + 6 * ((size_t)j0 * g.n_az + i1);
+    c.t10 = g.table + 6 * ((size_t)j1 * g.n_az + i0);
+    c.t11 = g.table + 6 * ((size_t)j1 * g.n_az + i1);
+    return c;
+}
+__device__ __forceinline__ double spad_value(const SpadCell &c, int k, double r2)
+{
+    return (c.w00 * __ldg(c.t00 + k) + c.w01 * __ldg(c.t01 + k) + c.w10 * __ldg(c.t10 + k) + c.w11 * __ldg(c.t11 + k)) * r2;
+}
+
+// Bilinear interpolant of the SPAD table at body-frame direction s and Sun
+// distance dist (AU; negative gives zeros): out = [F, T] scaled by 1/dist^2.
+__device__ __forceinline__ void spad_lookup(const SpadDev &g, const double *s, double dist, double out[6])
+{
+    if (dist < 0.0) {
+        for (int k = 0; k < 6; k++) out[k] = 0.0;
+        return;
+    }
+    const double az = atan2(s[1], s[0]);
+    const double el = atan2(s[2], hypot(s[0], s[1]));
+    const double u = (az - g.az0) * (g.n_az * 0.15915494309189535);  // cells of 2 pi / n_az
+    const SpadCell c = spad_cell(g, u, u / g.n_az, (el - g.el0) / g.d_el);
     const double r2 = 1.0 / (dist * dist);
-    for (int k = 0; k < 6; k++)
-        out[k] = (w00 * __ldg(t00 + k) + w01 * __ldg(t01 + k) + w10 * __ldg(t10 + k) + w11 * __ldg(t11 + k)) * r2;
+    for (int k = 0; k < 6; k++) out[k] = spad_value(c, k, r2);
 }
 
 // Propagation settings as seen by the device (from srp_prop_params).
@@ -373,6 +393,8 @@ struct PropState {
     int done, status, shadow, pad_;
     int central, attitude;     // per-trajectory force model and attitude law
     double q[4], mass;         // attitude quaternion, spacecraft mass (kg)
+    double imass;              // 1 / mass
+    double grav[3];            // gravity at the stage
     double Qm[9];              // rotation of the normalised q, row-major (fixed per trajectory)
     double rs_st[13][3];       // Sun position at every stage time of the current step
 };
