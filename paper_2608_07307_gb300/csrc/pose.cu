@@ -1,6 +1,6 @@
 // pose.cu -- per-evaluation geometry update (Sec. 4.4.2) and window bounds.
 //
-//   k_pose      a warp per evaluation slot, a lane per part: joint angles (Sun tracking,
+//   k_pose      a block per evaluation slot, a 16-lane group per part: joint angles (Sun tracking,
 //               commanded, or tracking + offset; clamped), part transforms
 //               composed down the kinematic tree (Sec. 4.4.1), image-plane
 //               basis, window accumulators reset.
@@ -17,38 +17,56 @@
 
 namespace srp {
 
-// Rotation by the angle whose cosine and sine are c, s about unit axis a.
-__device__ inline void rot_axis_cs(const double *a, double c, double s, double *R)
-{
-    const double k = 1.0 - c;
-    R[0] = c + k * a[0] * a[0];        R[1] = k * a[0] * a[1] - s * a[2]; R[2] = k * a[0] * a[2] + s * a[1];
-    R[3] = k * a[1] * a[0] + s * a[2]; R[4] = c + k * a[1] * a[1];        R[5] = k * a[1] * a[2] - s * a[0];
-    R[6] = k * a[2] * a[0] - s * a[1]; R[7] = k * a[2] * a[1] + s * a[0]; R[8] = c + k * a[2] * a[2];
-}
-
 constexpr double kPiPose = 3.14159265358979323846;
 
-__global__ void __launch_bounds__(32) k_pose(const SlotDesc *sd, const double *sun_dirs, const double *sun_dist,
-                                             double P0, int eval0, int S, SlotPose *pose)
+// Four warps a slot, a 16-lane group a part (the parts of a tree level together,
+// each reading its parent's transform from shared memory).  What the kernel costs is
+// the FP64 instructions its longest warp issues, 64 cycles each whatever the lanes:
+// matrix elements, vector components and the quotients of a division have a lane
+// each, and the image-plane basis is formed by the last warp beside the first
+// parts.  (One part a lane: 193 instructions a warp, 5.9 us a launch of one slot.)
+constexpr int kPoseThreads = 128;
+constexpr int kPoseGroup = 16;
+static_assert(kMaxParts <= 32, "a warp holds the parts' depths");
+
+__device__ __forceinline__ double group_shfl(double x, int j) { return __shfl_sync(0xffffffffu, x, j, kPoseGroup); }
+
+__global__ void __launch_bounds__(kPoseThreads) k_pose(const SlotDesc *sd, const double *sun_dirs,
+                                                       const double *sun_dist, double P0, int eval0, int S,
+                                                       SlotPose *pose)
 {
     pdl_enter();
-    // a warp per slot, a lane per part: the parts of one tree level are posed
-    // together (their FP64 chains overlap), each reading its parent's transform
-    // from shared memory
-    const int slot = blockIdx.x, lane = threadIdx.x;
+    const int slot = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (slot >= S) return;
     __shared__ double sM[kMaxParts][9], sT[kMaxParts][3];
+    __shared__ unsigned s_track, s_free;
     SlotPose &P = pose[slot];
     const MeshDev *mesh = sd[slot].mesh;
     const double *angles = sd[slot].angles;
     const int panel_mode = sd[slot].panel_mode;
     const int e = eval0 + slot;
     double s[3] = {sun_dirs[3 * e], sun_dirs[3 * e + 1], sun_dirs[3 * e + 2]};
-    const double sn = sqrt(s[0] * s[0] + s[1] * s[1] + s[2] * s[2]);
-    for (int k = 0; k < 3; k++) s[k] /= sn;
     const double dist = sun_dist ? sun_dist[e] : 1.0;
     const int skip = dist < 0.0 ? 1 : 0;  // a negative distance asks to skip this evaluation
-    if (lane == 0) {
+    const int np = mesh->n_parts;
+    // depth of each part in the kinematic tree (parents precede children), a part a lane
+    const int par_l = (lane < np && lane > 0) ? mesh->part[lane].parent : -1;
+    int depth = 0;
+    for (int q = par_l, it = 0; it < kMaxParts && __any_sync(0xffffffffu, q >= 0); it++) {
+        const int up = __shfl_sync(0xffffffffu, par_l, q >= 0 ? q : 0);
+        if (q >= 0) depth++;
+        q = q >= 0 ? up : -1;
+    }
+    const int levels = __reduce_max_sync(0xffffffffu, lane < np ? depth : 0);
+    const int j = lane & (kPoseGroup - 1), c3 = j % 3;
+    const int k1 = c3 == 2 ? 0 : c3 + 1, k2 = c3 == 0 ? 2 : c3 - 1;
+    const double sn = sqrt(s[0] * s[0] + s[1] * s[1] + s[2] * s[2]);
+    {
+        const double x = (c3 == 0 ? s[0] : c3 == 1 ? s[1] : s[2]) / sn;
+        for (int k = 0; k < 3; k++) s[k] = group_shfl(x, k);
+    }
+    if (threadIdx.x == 0) {
+        s_track = s_free = 0u;
         P.eval = e;
         P.flags = 0;
         P.s_norm = sn;
@@ -56,104 +74,128 @@ __global__ void __launch_bounds__(32) k_pose(const SlotDesc *sd, const double *s
         P.track_mask = 0;
         P.skip = skip;
     }
-    if (skip) return;
-    const int np = mesh->n_parts;
-    const int p = lane;
-    PartInfo pi{};
-    if (p < np) pi = mesh->part[p];
-    // depth of each part in the kinematic tree (parents precede children)
-    const int par = (p < np && p > 0) ? pi.parent : -1;
-    int depth = 0;
-    for (int q = par, it = 0; it < kMaxParts && __any_sync(0xffffffffu, q >= 0); it++) {
-        const int up = __shfl_sync(0xffffffffu, par, q >= 0 ? q : 0);
-        if (q >= 0) depth++;
-        q = q >= 0 ? up : -1;
+    if (skip) return;  // uniform over the block
+    if (warp == 0 && lane < 9) {  // the root
+        const double m = (lane % 4 == 0) ? 1.0 : 0.0;
+        sM[0][lane] = m;
+        P.M[0][lane] = m;
+        if (lane < 3) sT[0][lane] = P.T[0][lane] = 0.0;
     }
-    const int levels = __reduce_max_sync(0xffffffffu, p < np ? depth : 0);
-    bool track = false, freej = false;
-    for (int L = 0; L <= levels; L++) {
-        if (p < np && depth == L) {
-            double *M = sM[p], *T = sT[p];
-            if (p == 0) {
-                for (int k = 0; k < 9; k++) M[k] = (k % 4 == 0) ? 1.0 : 0.0;
-                T[0] = T[1] = T[2] = 0.0;
-            } else {
-                const double *Mq = sM[par], *Tq = sT[par];
-                // cosine and sine of the joint angle: from the tracking direction itself
-                // when the limits cannot clamp it (no FP64 transcendentals), else from the angle
-                double th = 0.0, cth = 1.0, sth = 0.0;
-                bool have_cs = false;
-                if (pi.movable) {
-                    if (panel_mode != SRP_PANELS_SET) {
-                        // Sun in the parent's current frame: Mq^T s
-                        double sl[3];
-                        for (int k = 0; k < 3; k++) sl[k] = Mq[k] * s[0] + Mq[3 + k] * s[1] + Mq[6 + k] * s[2];
-                        const double *a = pi.axis, *n0 = pi.n0;
-                        const double na = n0[0] * a[0] + n0[1] * a[1] + n0[2] * a[2];
-                        const double n[3] = {n0[0] - na * a[0], n0[1] - na * a[1], n0[2] - na * a[2]};
-                        const double b[3] = {a[1] * n[2] - a[2] * n[1], a[2] * n[0] - a[0] * n[2], a[0] * n[1] - a[1] * n[0]};
-                        const double x = n[0] * sl[0] + n[1] * sl[1] + n[2] * sl[2];
-                        const double y = b[0] * sl[0] + b[1] * sl[1] + b[2] * sl[2];
-                        track = !(x == 0.0 && y == 0.0);
-                        const bool plain = panel_mode == SRP_PANELS_TRACK || !angles;
-                        if (plain && pi.lim[0] <= -kPiPose && pi.lim[1] >= kPiPose && !(x < 0.0 && fabs(y) <= 1e-12 * -x)) {
-                            // atan2(y, x) lies strictly inside (-pi, pi): never clamped, always free
-                            const double r = sqrt(x * x + y * y);
-                            if (r > 0.0) { cth = x / r; sth = y / r; }
-                            have_cs = true;
-                            freej = true;
-                        }
-                        th = (x == 0.0 && y == 0.0) ? 0.0 : (have_cs ? 0.0 : atan2(y, x));
-                        if (panel_mode == SRP_PANELS_TRACK_OFFSET && angles) th += angles[p];
-                    } else {
-                        th = angles ? angles[p] : 0.0;
-                    }
-                    if (!have_cs) {
-                        if (th > pi.lim[0] && th < pi.lim[1]) freej = true;
-                        th = fmin(fmax(th, pi.lim[0]), pi.lim[1]);
-                        sincos(th, &sth, &cth);
-                    }
-                }
-                double R[9];
-                if (pi.movable) rot_axis_cs(pi.axis, cth, sth, R);
-                else for (int k = 0; k < 9; k++) R[k] = (k % 4 == 0) ? 1.0 : 0.0;
-                for (int i = 0; i < 3; i++)
-                    for (int j = 0; j < 3; j++)
-                        M[3 * i + j] = Mq[3 * i] * R[j] + Mq[3 * i + 1] * R[3 + j] + Mq[3 * i + 2] * R[6 + j];
-                const double *pv = pi.pivot;
-                double w[3];
-                for (int i = 0; i < 3; i++) w[i] = pv[i] - (R[3 * i] * pv[0] + R[3 * i + 1] * pv[1] + R[3 * i + 2] * pv[2]);
-                for (int i = 0; i < 3; i++) T[i] = Mq[3 * i] * w[0] + Mq[3 * i + 1] * w[1] + Mq[3 * i + 2] * w[2] + Tq[i];
+    if (warp == kPoseThreads / 32 - 1) {
+        // basis of the image plane around d = -s (Duff et al., JCGT 2017)
+        const double d[3] = {-s[0], -s[1], -s[2]};
+        const double sg = copysign(1.0, d[2]);
+        const double q = (lane == 1 ? P0 : -1.0) / (lane == 1 ? dist * dist : sg + d[2]);
+        const double a = __shfl_sync(0xffffffffu, q, 0), scale = __shfl_sync(0xffffffffu, q, 1);
+        const double b = d[0] * d[1] * a;
+        const double u[3] = {1.0 + sg * d[0] * d[0] * a, sg * b, -sg * d[0]};
+        const double v[3] = {b, sg + d[1] * d[1] * a, -d[1]};
+        if (lane == 0) {
+            for (int k = 0; k < 3; k++) {
+                P.u[k] = u[k];
+                P.v[k] = v[k];
+                P.d[k] = d[k];
+                P.s[k] = s[k];
+                P.wmin_bits[k] = dbl_to_ord(INFINITY);
+                P.wmax_bits[k] = dbl_to_ord(-INFINITY);
             }
-            for (int k = 0; k < 9; k++) P.M[p][k] = M[k];
-            for (int k = 0; k < 3; k++) P.T[p][k] = T[k];
+            P.scale = scale;
         }
-        __syncwarp();
     }
-    const unsigned track_mask = __ballot_sync(0xffffffffu, track);
-    const unsigned free_mask = __ballot_sync(0xffffffffu, freej);
-    if (lane != 0) return;
-    P.track_mask = track_mask;
-    P.free_mask = free_mask;
-    // basis of the image plane around d = -s (Duff et al., JCGT 2017)
-    double d[3] = {-s[0], -s[1], -s[2]};
-    double sg = copysign(1.0, d[2]);
-    double a = -1.0 / (sg + d[2]);
-    double b = d[0] * d[1] * a;
-    P.u[0] = 1.0 + sg * d[0] * d[0] * a; P.u[1] = sg * b; P.u[2] = -sg * d[0];
-    P.v[0] = b; P.v[1] = sg + d[1] * d[1] * a; P.v[2] = -d[1];
-    for (int k = 0; k < 3; k++) { P.d[k] = d[k]; P.s[k] = s[k]; }
-    for (int k = 0; k < 3; k++) {
-        P.wmin_bits[k] = dbl_to_ord(INFINITY);
-        P.wmax_bits[k] = dbl_to_ord(-INFINITY);
+    __syncthreads();
+    for (int L = 1; L <= levels; L++) {
+        for (int p0 = 2 * warp; p0 < np; p0 += kPoseThreads / kPoseGroup) {
+            const int p = p0 + (lane >> 4);
+            const bool act = __shfl_sync(0xffffffffu, depth, min(p, np - 1)) == L && p < np;
+            if (!__any_sync(0xffffffffu, act)) continue;
+            // (the warp's other part is worked along, and not stored, when it is of another level)
+            const int pc = act ? p : 0;
+            const PartInfo &pi = mesh->part[pc];
+            const int par = act ? pi.parent : 0;
+            const double *Mq = sM[par], *Tq = sT[par];
+            const double axis[3] = {pi.axis[0], pi.axis[1], pi.axis[2]};
+            const bool movable = act && pi.movable;
+            // cosine and sine of the joint angle: from the tracking direction itself
+            // when the limits cannot clamp it (no FP64 transcendentals), else from the angle
+            double th = 0.0, cth = 1.0, sth = 0.0;
+            bool have_cs = false, track = false, freej = false;
+            if (panel_mode != SRP_PANELS_SET) {  // uniform over the block
+                // lanes 0-2: the Sun in the parent's current frame, Mq^T s; lane 3: n0 . axis
+                const bool m3 = j < 3;
+                const double dt = (m3 ? Mq[c3] : pi.n0[0]) * (m3 ? s[0] : axis[0]) +
+                                  (m3 ? Mq[3 + c3] : pi.n0[1]) * (m3 ? s[1] : axis[1]) +
+                                  (m3 ? Mq[6 + c3] : pi.n0[2]) * (m3 ? s[2] : axis[2]);
+                double sl[3], n[3], b[3];
+                for (int k = 0; k < 3; k++) sl[k] = group_shfl(dt, k);
+                const double na = group_shfl(dt, 3);
+                const double nc = pi.n0[c3] - na * pi.axis[c3];
+                for (int k = 0; k < 3; k++) n[k] = group_shfl(nc, k);
+                const double bc = pi.axis[k1] * (k2 == 0 ? n[0] : k2 == 1 ? n[1] : n[2]) -
+                                  pi.axis[k2] * (k1 == 0 ? n[0] : k1 == 1 ? n[1] : n[2]);
+                for (int k = 0; k < 3; k++) b[k] = group_shfl(bc, k);
+                const bool second = j == 1;
+                const double xy = (second ? b[0] : n[0]) * sl[0] + (second ? b[1] : n[1]) * sl[1] +
+                                  (second ? b[2] : n[2]) * sl[2];
+                const double x = group_shfl(xy, 0), y = group_shfl(xy, 1);
+                track = movable && !(x == 0.0 && y == 0.0);
+                const bool plain = panel_mode == SRP_PANELS_TRACK || !angles;
+                // atan2(y, x) strictly inside (-pi, pi): never clamped, always free
+                have_cs = movable && plain && pi.lim[0] <= -kPiPose && pi.lim[1] >= kPiPose &&
+                          !(x < 0.0 && fabs(y) <= 1e-12 * -x);
+                if (__any_sync(0xffffffffu, have_cs)) {
+                    const double r = sqrt(x * x + y * y);
+                    const double q = (second ? y : x) / (r > 0.0 ? r : 1.0);
+                    const double c = group_shfl(q, 0), sq = group_shfl(q, 1);
+                    if (have_cs && r > 0.0) { cth = c; sth = sq; }
+                }
+                freej = have_cs;
+                if (movable && !have_cs) {
+                    th = (x == 0.0 && y == 0.0) ? 0.0 : atan2(y, x);
+                    if (panel_mode == SRP_PANELS_TRACK_OFFSET && angles) th += angles[p];
+                }
+            } else if (movable) {
+                th = angles ? angles[p] : 0.0;
+            }
+            if (movable && !have_cs) {
+                if (th > pi.lim[0] && th < pi.lim[1]) freej = true;
+                th = fmin(fmax(th, pi.lim[0]), pi.lim[1]);
+                sincos(th, &sth, &cth);
+            }
+            __syncwarp();
+            // rotation about the axis by that angle, element (r, c) in lane 3 r + c of the group
+            const int rr = j < 9 ? j / 3 : 0;
+            const double k = 1.0 - cth;
+            const double ar = pi.axis[rr], ac = pi.axis[c3];
+            const double ss = (c3 - rr + 3) % 3 == 1 ? sth : -sth;
+            const double diag = cth + k * ar * ac;
+            const double off = k * ar * ac - ss * pi.axis[rr == c3 ? 0 : 3 - rr - c3];
+            const double R = !movable ? (rr == c3 ? 1.0 : 0.0) : rr == c3 ? diag : off;
+            const double m = Mq[3 * rr] * group_shfl(R, c3) + Mq[3 * rr + 1] * group_shfl(R, 3 + c3) +
+                             Mq[3 * rr + 2] * group_shfl(R, 6 + c3);
+            const double *pv = pi.pivot;
+            const double wc = pv[c3] - (group_shfl(R, 3 * c3) * pv[0] + group_shfl(R, 3 * c3 + 1) * pv[1] +
+                                        group_shfl(R, 3 * c3 + 2) * pv[2]);
+            const double t = Mq[3 * c3] * group_shfl(wc, 0) + Mq[3 * c3 + 1] * group_shfl(wc, 1) +
+                             Mq[3 * c3 + 2] * group_shfl(wc, 2) + Tq[c3];
+            if (act) {
+                if (j < 9) sM[p][j] = P.M[p][j] = m;
+                if (j < 3) sT[p][j] = P.T[p][j] = t;
+                if (j == 0 && track) atomicOr(&s_track, 1u << p);
+                if (j == 0 && freej) atomicOr(&s_free, 1u << p);
+            }
+        }
+        __syncthreads();
     }
-    P.scale = P0 / (dist * dist);
+    if (threadIdx.x == 0) {
+        P.track_mask = s_track;
+        P.free_mask = s_free;
+    }
 }
 
 cudaError_t launch_pose(const SlotDesc *sd, const double *sun_dirs, const double *sun_dist, double P0, int eval0,
                         int S, SlotPose *pose, cudaStream_t st)
 {
-    return launch_chained(k_pose, dim3(S), dim3(32), 0, st, sd, sun_dirs, sun_dist, P0, eval0, S, pose);
+    return launch_chained(k_pose, dim3(S), dim3(kPoseThreads), 0, st, sd, sun_dirs, sun_dist, P0, eval0, S, pose);
 }
 
 // ------------------------------------------------------------- vertices

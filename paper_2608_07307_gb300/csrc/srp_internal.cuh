@@ -222,7 +222,7 @@ struct TraceArgs {
     int n_blocks_x;              // stride of the per-tile arrays: the largest tile count of a slot
     float *partials;             // [S][n_blocks_x][6] force and torque per tile (FP32 tile sums)
     unsigned *pcounts;           // [S][n_blocks_x][kCnt] counts 6..19 per tile
-    double *partials1;           // [S][kRed1][kPart] first-level sums of the tile partials
+    double *partials1;           // [S][kRed1][kPart] first-level sums of the tile partials (counts: bits of 64-bit integers)
     unsigned *red_ticket;        // [S] first-level blocks done (the last one adds their sums); reset by the frame kernel
     int *amb_list;               // [S][n_blocks_x][kTileRays] rays handed to the FP64 path, per tile
     int *amb_count;              // [S][n_blocks_x]

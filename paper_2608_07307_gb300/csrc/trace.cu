@@ -197,7 +197,11 @@ __global__ void k_frame(TraceArgs a)
     const int n_tris = m->n_tris;
     const float4 *node_static = m->node_static, *tri_static = m->tri_static;
     const double *rest64 = m->rest64;
-    double wlo[3], whi[3], u3[3], v3[3], d3[3], cref[3], Rm = 0.0, pad = 0.0;
+    // a component a lane (of three): an FP64 instruction costs the warp the same for one lane or all
+    const int c3 = lane % 3;
+    const double lo = ord_to_dbl(P.wmin_bits[c3]), hi = ord_to_dbl(P.wmax_bits[c3]);
+    const double u3 = P.u[c3], v3 = P.v[c3], d3 = P.d[c3], cref = m->c_ref[c3];
+    double Rm = 0.0, pad = 0.0;
     int n_mats = 0;
     const float2 *mat32 = nullptr;
     const double *mat64 = nullptr;
@@ -205,12 +209,6 @@ __global__ void k_frame(TraceArgs a)
     const int *tri_vidx = nullptr;
     const int2 *grp = nullptr;
     if (lane == 0) {
-        for (int k = 0; k < 3; k++) {
-            wlo[k] = ord_to_dbl(P.wmin_bits[k]);
-            whi[k] = ord_to_dbl(P.wmax_bits[k]);
-            u3[k] = P.u[k]; v3[k] = P.v[k]; d3[k] = P.d[k];
-            cref[k] = m->c_ref[k];
-        }
         Rm = m->R;
         pad = m->pad;
         n_mats = m->n_mats;
@@ -259,30 +257,35 @@ __global__ void k_frame(TraceArgs a)
             pv.box_src = box_static;
         }
     }
-    if (lane != 0) return;
-    const double umin = wlo[0], umax = whi[0], vmin = wlo[1], vmax = whi[1], wmin = wlo[2], wmax = whi[2];
-    const double Du = umax - umin, Dv = vmax - vmin, Dw = wmax - wmin;
+    const auto all = [](double x, int l) { return __shfl_sync(0xffffffffu, x, l); };
+    const double umin = all(lo, 0), umax = all(hi, 0), vmin = all(lo, 1), vmax = all(hi, 1), wmin = all(lo, 2),
+                 wmax = all(hi, 2);
+    const double D3 = hi - lo;
+    const double Du = all(D3, 0), Dv = all(D3, 1), Dw = all(D3, 2);
     const double Lw = sqrt(Du * Du + Dv * Dv + Dw * Dw);
     const double eps = a.eps_rel * Lw;
+    const double qn = (lane == 0 ? Du : lane == 1 ? Dv : 1.0) / N;  // the pixel's sides and 1 / N
+    const double DuN = all(qn, 0), DvN = all(qn, 1), rN = all(qn, 2);
+    const double w0 = wmin - kStandoff;
+    const double o3 = umin * u3 + vmin * v3 + w0 * d3;
+    if (lane < 3) {
+        B.org[lane] = (float)o3;
+        B.du[lane] = (float)(DuN * u3);
+        B.dv[lane] = (float)(DvN * v3);
+        B.dir[lane] = (float)d3;
+        B.u[lane] = u3; B.v[lane] = v3; B.d[lane] = d3;
+        B.c_ref[lane] = cref;
+        B.cref32[lane] = (float)cref;
+    }
+    if (lane != 0) return;
     B.umin = umin; B.vmin = vmin; B.wmin = wmin;
-    B.rN = (N & (N - 1)) == 0 ? 1.0 / N : 0.0;
+    B.rN = (N & (N - 1)) == 0 ? rN : 0.0;
     B.Du = Du; B.Dv = Dv;
     B.Lw = Lw;
     B.eps = eps;
     B.eps32 = (float)eps;
-    const double w0 = wmin - kStandoff;
-    for (int k = 0; k < 3; k++) {
-        double o = umin * u3[k] + vmin * v3[k] + w0 * d3[k];
-        B.org[k] = (float)o;
-        B.du[k] = (float)(Du / N * u3[k]);
-        B.dv[k] = (float)(Dv / N * v3[k]);
-        B.dir[k] = (float)d3[k];
-        B.u[k] = u3[k]; B.v[k] = v3[k]; B.d[k] = d3[k];
-        B.c_ref[k] = cref[k];
-        B.cref32[k] = (float)cref[k];
-    }
     B.umin32 = (float)umin; B.vmin32 = (float)vmin;
-    B.du32 = (float)(Du / N); B.dv32 = (float)(Dv / N);
+    B.du32 = (float)DuN; B.dv32 = (float)DvN;
     B.rdu32 = 1.0f / B.du32; B.rdv32 = 1.0f / B.dv32;
     B.w0_32 = (float)w0;
     const double u = 5.9604644775390625e-8;
@@ -1315,22 +1318,26 @@ __device__ inline double warp_sum(double x)
     return x;
 }
 
-// Block-wide FP64 sum of v[0..kPart) into out[0..kPart) (fixed order).
-__device__ void block_sum(const double *v, double *out)
+// The warp's sums of six FP64 values by warp_sum's tree, each step halving what a
+// lane carries: 8 additions instead of 30 (an FP64 instruction holds the pipe for 64
+// cycles a warp).  The sum of value sum6_value(lane) is returned in lanes 0, 4, 8, 16, 20, 24.
+__device__ __forceinline__ int sum6_value(int lane)
 {
-    __shared__ double red[kPart][32];
-    int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int k = 0; k < kPart; k++) {
-        double x = warp_sum(v[k]);
-        if (lane == 0) red[k][w] = x;
-    }
-    __syncthreads();
-    if (threadIdx.x < kPart) {
-        double x = 0.0;
-        for (int i = 0; i < (int)(blockDim.x >> 5); i++) x += red[threadIdx.x][i];
-        out[threadIdx.x] = x;
-    }
-    __syncthreads();
+    return (lane & 16 ? 3 : 0) + (lane & 4 ? 1 : lane & 8 ? 2 : 0);
+}
+__device__ __forceinline__ bool sum6_holds(int lane) { return (lane & 3) == 0 && (lane & 12) != 12; }
+__device__ __forceinline__ double warp_sum6(const double *v, int lane)
+{
+    const auto other = [](double x, int o) { return __shfl_xor_sync(0xffffffffu, x, o); };
+    const bool h16 = lane & 16, h8 = lane & 8, h4 = lane & 4;
+    double a[3];
+    for (int k = 0; k < 3; k++) a[k] = (h16 ? v[3 + k] : v[k]) + other(h16 ? v[k] : v[3 + k], 16);
+    const double b0 = (h8 ? a[2] : a[0]) + other(h8 ? a[0] : a[2], 8);
+    const double b1 = a[1] + other(a[1], 8);
+    double c = (h4 ? b1 : b0) + other(h4 ? b0 : b1, 4);
+    c += other(c, 2);
+    c += other(c, 1);
+    return c;
 }
 
 // Slot of flattened trace block g: the last slot whose first block is <= g.
@@ -2946,8 +2953,10 @@ __global__ void __launch_bounds__(256) k_reduce1(TraceArgs a, int eval0, double 
     const int kc = a.count ? kCnt : 7;  // the trace writes the traversal counters only when counting
     int mine = 0;
     for (int t = t0 + (int)threadIdx.x; t < t1; t += blockDim.x) {
+        const float2 *pp = reinterpret_cast<const float2 *>(a.partials + (base + t) * 6);
+        const float2 p2[3] = {pp[0], pp[1], pp[2]};
         for (int k = 0; k < 6; k++) {
-            const float p = a.partials[(base + t) * 6 + k];
+            const float p = k & 1 ? p2[k >> 1].y : p2[k >> 1].x;
             if (mode == 0) f[k] += (double)p;
             else if (mode == 1) comp_add(f32[k], p);
             else f32[k].hi = __fadd_rn(f32[k].hi, p);
@@ -2986,18 +2995,14 @@ __global__ void __launch_bounds__(256) k_reduce1(TraceArgs a, int eval0, double 
     __shared__ Comp32 r32[6][256];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (mode == 0) {
-        for (int k = 0; k < 6; k++) {
-            const double x = warp_sum(f[k]);
-            if (lane == 0) rf[k][w] = x;
-        }
+        const double x = warp_sum6(f, lane);
+        if (sum6_holds(lane)) rf[sum6_value(lane)][w] = x;
     } else {
         for (int k = 0; k < 6; k++) r32[k][threadIdx.x] = f32[k];
     }
     for (int k = 0; k < kCnt; k++) {
         // only the live counts (kc is uniform over the launch)
-        unsigned x = c[k];
-        if (k < kc)
-            for (int o = 16; o; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+        const unsigned x = k < kc ? __reduce_add_sync(0xffffffffu, c[k]) : c[k];
         if (lane == 0) rc[k][w] = x;
     }
     __syncthreads();
@@ -3019,7 +3024,7 @@ __global__ void __launch_bounds__(256) k_reduce1(TraceArgs a, int eval0, double 
     } else if (threadIdx.x < kPart) {
         unsigned long long x = 0ull;
         for (int q = 0; q < nw; q++) x += rc[threadIdx.x - 6][q];
-        out[threadIdx.x] = (double)x;
+        out[threadIdx.x] = __longlong_as_double((long long)x);  // (an integer's bits)
     }
     if (!fuse) return;
     // the last of the slot's blocks to finish adds the first-level sums, in
@@ -3034,83 +3039,77 @@ __global__ void __launch_bounds__(256) k_reduce1(TraceArgs a, int eval0, double 
     final_reduce(a, s, eval0, force, torque, err_flags, stats_accum, true);
 }
 
-// The second level for slot s: its kRed1 first-level sums added in block order
-// (FP64; the FP32 modes add them again in FP32), the diffuse blocks' sums, the
-// pixel-area scale, the stores.  Threads below kRed1 of the calling block hold
-// the sums (whole warps); `cg` reads what other blocks of the same launch wrote
-// through L2.  stats_accum[16]: 0 evals, 1 rays, 2 refined rays, 3 segments,
-// 4..8 hits per segment, 9 nodes, 10 triangles, 11 box tests, 12..15 hand-offs
-// by cause.
+// The second level for slot s: its kRed1 first-level sums added by warps in a
+// fixed tree (FP64; the FP32 modes add them again in FP32, in block order), the
+// diffuse blocks' sums in block order, the pixel-area scale, the stores.  The
+// calling block has kRed1 threads at least; `cg` reads what other blocks of the
+// same launch wrote through L2.  The first warps sum the forces, the last one forms
+// the scale beside them, and the counts (whole numbers) are added by every warp:
+// the FP64 chain after the last block's arrival is 8 + kRed1 / 32 additions and a
+// product (100 additions a warp and a serial tail, 18 us a launch of one slot, before).
+// stats_accum[16]: 0 evals, 1 rays, 2 refined rays, 3 segments, 4..8 hits per segment,
+// 9 nodes, 10 triangles, 11 box tests, 12..15 hand-offs by cause.
 __device__ void final_reduce(const TraceArgs &a, int s, int eval0, double *force, double *torque, int *err_flags,
                              unsigned long long *stats_accum, bool cg)
 {
-    // what the last step needs, loaded before the sums (a load is not moved across the barriers)
-    const SlotPose &P = a.pose[s];
-    double Du = 0.0, Dv = 0.0, scale = 0.0;
-    int N = 0, pflags = 0;
-    if (threadIdx.x == 0) {
-        Du = ord_to_dbl(P.wmax_bits[0]) - ord_to_dbl(P.wmin_bits[0]);
-        Dv = ord_to_dbl(P.wmax_bits[1]) - ord_to_dbl(P.wmin_bits[1]);
-        scale = P.scale;
-        pflags = cg ? __ldcg(&P.flags) : P.flags;
-        N = a.sd[s].N;
+    __shared__ double red2[6][kRed1 / 32];
+    __shared__ double s_scale;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = (int)(blockDim.x >> 5);
+    const auto first = [&](int b, int k) {
+        const double *src = a.partials1 + ((size_t)s * kRed1 + b) * kPart + k;
+        return cg ? __ldcg(src) : *src;
+    };
+    if (w < kRed1 / 32) {
+        double v[6];
+        for (int k = 0; k < 6; k++) v[k] = first(threadIdx.x, k);
+        const double x = warp_sum6(v, lane);
+        if (sum6_holds(lane)) red2[sum6_value(lane)][w] = x;
     }
-    __shared__ double red2[kPart][kRed1 / 32];
-    __shared__ double red[kPart];
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (threadIdx.x < kRed1) {
-        const double *src = a.partials1 + ((size_t)s * kRed1 + threadIdx.x) * kPart;
-        for (int k = 0; k < kPart; k++) {
-            const double x = warp_sum(cg ? __ldcg(src + k) : src[k]);
-            if (lane == 0) red2[k][w] = x;
-        }
-    }
-    __syncthreads();
-    if (threadIdx.x < kPart) {
-        double x = 0.0;
-        for (int q = 0; q < kRed1 / 32; q++) x += red2[threadIdx.x][q];
-        red[threadIdx.x] = x;
-    }
-    __syncthreads();
-    if (threadIdx.x != 0) return;
-    if (a.sum_mode != 0) {
-        // the FP32 modes: the first-level sums again, in order, in FP32
-        for (int k = 0; k < 6; k++) {
-            Comp32 x{0.0f, 0.0f};
-            for (int b = 0; b < kRed1; b++) {
-                const double *src = a.partials1 + ((size_t)s * kRed1 + b) * kPart + k;
-                const float p = (float)(cg ? __ldcg(src) : *src);
-                if (a.sum_mode == 1) comp_add(x, p);
-                else x.hi = __fadd_rn(x.hi, p);
+    if (w == nw - 1) {
+        const SlotPose &P = a.pose[s];
+        const int N = a.sd[s].N;
+        const double Du = ord_to_dbl(P.wmax_bits[0]) - ord_to_dbl(P.wmin_bits[0]);
+        const double Dv = ord_to_dbl(P.wmax_bits[1]) - ord_to_dbl(P.wmin_bits[1]);
+        const double sc = P.scale * (Du * Dv) / ((double)N * (double)N);
+        if (lane == 0) {
+            s_scale = sc;
+            const int pflags = cg ? __ldcg(&P.flags) : P.flags;
+            if (pflags) atomicOr(err_flags, pflags);
+            if (stats_accum) {
+                atomicAdd(&stats_accum[0], 1ull);
+                atomicAdd(&stats_accum[1], (unsigned long long)N * (unsigned long long)N);
             }
-            if (a.n_diffuse > 0)
-                for (int b = 0; b < kDiffBlocks; b++) {
-                    const float p = (float)a.dpart[((size_t)s * kDiffBlocks + b) * 6 + k];
-                    if (a.sum_mode == 1) comp_add(x, p);
-                    else x.hi = __fadd_rn(x.hi, p);
-                }
-            red[k] = (double)comp_value(x);
         }
-    } else if (a.n_diffuse > 0) {
-        for (int b = 0; b < kDiffBlocks; b++)
-            for (int k = 0; k < 6; k++) red[k] += a.dpart[((size_t)s * kDiffBlocks + b) * 6 + k];
     }
-    const double sc = scale * (Du * Dv) / ((double)N * (double)N);
-    const int e = eval0 + s;
-    for (int k = 0; k < 3; k++) {
-        force[3 * e + k] = red[k] * sc;
-        torque[3 * e + k] = red[3 + k] * sc;
-    }
-    if (pflags) atomicOr(err_flags, pflags);
     if (stats_accum) {
-        atomicAdd(&stats_accum[0], 1ull);
-        atomicAdd(&stats_accum[1], (unsigned long long)N * (unsigned long long)N);
-        atomicAdd(&stats_accum[2], (unsigned long long)red[6]);
-        atomicAdd(&stats_accum[3], (unsigned long long)red[7]);
-        for (int k = 0; k < 5; k++) atomicAdd(&stats_accum[4 + k], (unsigned long long)red[8 + k]);
-        for (int k = 0; k < 3; k++) atomicAdd(&stats_accum[9 + k], (unsigned long long)red[13 + k]);
-        for (int k = 0; k < 4; k++) atomicAdd(&stats_accum[12 + k], (unsigned long long)red[16 + k]);
+        for (int k = nw - 1 - w; k < kCnt; k += nw) {
+            unsigned long long x = 0ull;
+            for (int b = lane; b < kRed1; b += 32) x += (unsigned long long)__double_as_longlong(first(b, 6 + k));
+            for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+            if (lane == 0 && x) atomicAdd(&stats_accum[2 + k], x);
+        }
     }
+    __syncthreads();
+    if (threadIdx.x >= 6) return;
+    const int k = threadIdx.x;
+    double x = 0.0;
+    if (a.sum_mode == 0) {
+        for (int q = 0; q < kRed1 / 32; q++) x += red2[k][q];
+        if (a.n_diffuse > 0)
+            for (int b = 0; b < kDiffBlocks; b++) x += a.dpart[((size_t)s * kDiffBlocks + b) * 6 + k];
+    } else {
+        // the FP32 modes: the first-level sums again, in order, in FP32
+        Comp32 y{0.0f, 0.0f};
+        const auto add = [&](float p) {
+            if (a.sum_mode == 1) comp_add(y, p);
+            else y.hi = __fadd_rn(y.hi, p);
+        };
+        for (int b = 0; b < kRed1; b++) add((float)first(b, k));
+        if (a.n_diffuse > 0)
+            for (int b = 0; b < kDiffBlocks; b++) add((float)a.dpart[((size_t)s * kDiffBlocks + b) * 6 + k]);
+        x = (double)comp_value(y);
+    }
+    (k < 3 ? force : torque)[3 * (eval0 + s) + k % 3] = x * s_scale;
 }
 
 // The second level as its own launch (after the diffuse rays), a block per slot.
