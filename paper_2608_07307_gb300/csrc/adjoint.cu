@@ -5,9 +5,9 @@
 // angles (hence the joint offsets and, through Sun tracking, the Sun
 // direction), the Sun direction and the Sun distance (Sec. 4.3, 4.4.2, 6.1).
 //
-//   k_adj_window  blocks per slot over the posed vertices, extreme along u and v
-//                 (k_adj_window_merge: the blocks' extremes in block order)
-//                 (lowest vertex index among equal projections).
+//   k_adj_window  blocks per slot over the posed vertices: those at the window's
+//                 bounds along u and v (lowest vertex index among equal projections,
+//                 a block's; the later kernels take the lowest of the blocks').
 //   k_adj_rays    grid-stride over the rays of every slot: per ray, the
 //                 segments are replayed forward in FP32 from the recorded hits,
 //                 then swept backward; cotangents of the ray direction, the
@@ -27,6 +27,8 @@
 // per segment f = w [(1 - rho_s) d - 2 (rho_s c + rho_d / 3) n_f],
 // T = scale * A_pix * sum (x - c_ref) x f.
 #include <math.h>
+
+#include <limits.h>
 
 #include <algorithm>
 
@@ -62,12 +64,6 @@ __device__ inline V3 mat_tmul(const double *M, V3 x)
             M[2] * x.x + M[5] * x.y + M[8] * x.z};
 }
 
-__device__ inline double wsum(double x)
-{
-    for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
-    return x;
-}
-
 // posed FP64 position of (re-indexed) vertex v of a slot
 __device__ inline V3 vertex(const MeshDev &m, const SlotBufs &sb, int v)
 {
@@ -76,89 +72,62 @@ __device__ inline V3 vertex(const MeshDev &m, const SlotBufs &sb, int v)
     return ld3(sb.vert64 + (size_t)(v - pi.vert_begin + pi.dyn_vert_off) * 3);
 }
 
-// Add val[0..n) of the lanes holding `key` (>= 0) into row[key * n ..], for
-// every distinct key in the warp: masked butterfly sums, one writer (lane 0).
-template <int n>
-__device__ inline void warp_scatter(int key, const double *val, double *row)
-{
-    unsigned todo = __ballot_sync(kFull, key >= 0);
-    while (todo) {
-        int k = __shfl_sync(kFull, key, __ffs(todo) - 1);
-        bool mine = key == k;
-        double sum[n];
-#pragma unroll
-        for (int c = 0; c < n; c++) sum[c] = wsum(mine ? val[c] : 0.0);
-        if ((threadIdx.x & 31) == 0) {
-#pragma unroll
-            for (int c = 0; c < n; c++) row[k * n + c] += sum[c];
-        }
-        todo &= ~__ballot_sync(kFull, mine);
-    }
-}
-
 // ------------------------------------------------------------- window
+// The window bounds are the exact extremes of the projections that the vertex
+// kernel stored, so the search is for equal bits: no FP64 arithmetic (14 us a launch
+// and 8 for the merge of its blocks as a search by FP64 comparisons).
 __global__ void __launch_bounds__(kAdjThreads) k_adj_window(AdjArgs a)
 {
+    pdl_enter();
     const int s = blockIdx.y, b = blockIdx.x, G = gridDim.x;
     const SlotPose &P = a.pose[s];
     if (P.skip) return;
     const MeshDev &m = *a.sd[s].mesh;
     const SlotBufs &sb = a.sd[s].sb;
-    V3 u = ld3(P.u), v = ld3(P.v);
-    double best[4] = {INFINITY, -INFINITY, INFINITY, -INFINITY};
-    int id[4] = {-1, -1, -1, -1};
-    for (int k = b * blockDim.x + threadIdx.x; k < m.n_verts; k += G * blockDim.x) {  // ascending k per thread
-        V3 x = vertex(m, sb, k);
-        double pu = dot(u, x), pv = dot(v, x);
-        if (pu < best[0]) { best[0] = pu; id[0] = k; }
-        if (pu > best[1]) { best[1] = pu; id[1] = k; }
-        if (pv < best[2]) { best[2] = pv; id[2] = k; }
-        if (pv > best[3]) { best[3] = pv; id[3] = k; }
-    }
-    __shared__ double sv[4][kAdjThreads];
-    __shared__ int si[4][kAdjThreads];
-    for (int c = 0; c < 4; c++) { sv[c][threadIdx.x] = best[c]; si[c][threadIdx.x] = id[c]; }
+    __shared__ int low[4];
+    if (threadIdx.x < 4) low[threadIdx.x] = INT_MAX;
     __syncthreads();
-    for (int h = kAdjThreads / 2; h > 0; h >>= 1) {
-        if ((int)threadIdx.x < h) {
-            for (int c = 0; c < 4; c++) {
-                double b0 = sv[c][threadIdx.x], b1 = sv[c][threadIdx.x + h];
-                int i0 = si[c][threadIdx.x], i1 = si[c][threadIdx.x + h];
-                bool take = (c & 1) ? (b1 > b0) : (b1 < b0);
-                if (i1 >= 0 && (i0 < 0 || take || (b1 == b0 && i1 < i0))) {
-                    sv[c][threadIdx.x] = b1;
-                    si[c][threadIdx.x] = i1;
-                }
+    // the two zeros are one bound
+    const unsigned long long zero = dbl_to_ord(0.0);
+    const auto key = [zero](unsigned long long o) { return o == zero - 1 ? zero : o; };
+    const unsigned long long bound[4] = {key(P.wmin_bits[0]), key(P.wmax_bits[0]), key(P.wmin_bits[1]),
+                                         key(P.wmax_bits[1])};
+    const int stride = G * blockDim.x;
+    for (int k = b * blockDim.x + threadIdx.x; k < m.n_verts; k += stride) {
+        const double *x = sb.vview64 + 3 * (size_t)k;
+        const unsigned long long pu = key(dbl_to_ord(x[0])), pv = key(dbl_to_ord(x[1]));
+        for (int c = 0; c < 4; c++)
+            if ((c < 2 ? pu : pv) == bound[c]) atomicMin(&low[c], k);
+    }
+    if (a.records) {
+        // the records the rays read, of the dynamic parts (those of the static parts are the mesh's)
+        for (int q = b * blockDim.x + threadIdx.x; q < m.n_dyn_tris; q += stride) {
+            const int4 tv = m.tri_v4[m.n_static_tris + q];
+            float4 *rec = sb.tri + 3 * (size_t)q;
+            const int id[3] = {tv.x, tv.y, tv.z};
+            for (int c = 0; c < 3; c++) {
+                const V3 x = vertex(m, sb, id[c]);
+                rec[c] = make_float4((float)x.x, (float)x.y, (float)x.z,
+                                     c == 0 ? __int_as_float(m.tri_orig[m.n_static_tris + q])
+                                     : c == 1 ? __uint_as_float(m.tri_mat[m.n_static_tris + q]) : 0.0f);
             }
         }
-        __syncthreads();
     }
-    if (threadIdx.x < 4) {
-        const size_t o = ((size_t)s * G + b) * 4 + threadIdx.x;
-        a.win_val[o] = sv[threadIdx.x][0];
-        a.win_pid[o] = si[threadIdx.x][0];
-    }
+    __syncthreads();
+    if (threadIdx.x < 4) a.win_pid[((size_t)s * G + b) * 4 + threadIdx.x] = low[threadIdx.x];
 }
 
-// The blocks' extremes of a slot merged in block order: the extreme value, the
-// lowest vertex id among equal values (the single-block search's result).
-__global__ void k_adj_window_merge(AdjArgs a, int G)
+int win_blocks(const AdjArgs &a)
 {
-    const int s = blockIdx.x, c = threadIdx.x;
-    if (a.pose[s].skip || c >= 4) return;
-    double best = (c & 1) ? -INFINITY : INFINITY;
-    int id = -1;
-    for (int b = 0; b < G; b++) {
-        const size_t o = ((size_t)s * G + b) * 4 + c;
-        const double v = a.win_val[o];
-        const int i = a.win_pid[o];
-        const bool take = (c & 1) ? (v > best) : (v < best);
-        if (i >= 0 && (id < 0 || take || (v == best && i < id))) {
-            best = v;
-            id = i;
-        }
-    }
-    a.win_ids[4 * s + c] = id;
+    const int items = std::max(a.n_verts, a.records ? a.n_dyn_tris : 0);
+    return std::max(1, std::min(kAdjWinBlocks, (items + 4 * kAdjThreads - 1) / (4 * kAdjThreads)));
+}
+
+// The window's extreme vertex c (0..3) of slot s: the lowest of its G <= 32 blocks', by a warp.
+__device__ __forceinline__ int window_vertex(const AdjArgs &a, int s, int c, int G)
+{
+    const int lane = threadIdx.x & 31;
+    return __reduce_min_sync(kFull, lane < G ? a.win_pid[((size_t)s * G + lane) * 4 + c] : INT_MAX);
 }
 
 // --------------------------------------------------------------- rays
@@ -177,36 +146,57 @@ __device__ inline F3 &operator+=(F3 &a, F3 b) { a.x += b.x; a.y += b.y; a.z += b
 __device__ inline float dot(F3 a, F3 b) { return a.x * b.x + a.y * b.y + a.z * b.z; }
 __device__ inline F3 cross(F3 a, F3 b) { return {a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x}; }
 
-__device__ inline float wsumf(float x)
+// The FP32 record of a sorted triangle: its posed vertices, rounded from FP64 (the
+// material pair in the second word's w).
+struct Tri32 {
+    F3 A, B, C;
+    unsigned mat;
+};
+__device__ __forceinline__ Tri32 tri32(const MeshDev &m, const SlotBufs &sb, int tri)
 {
-    for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
-    return x;
+    const int q = tri - m.n_static_tris;
+    const float4 *r = q < 0 ? m.tri_static + 3 * (size_t)tri : sb.tri + 3 * (size_t)q;
+    const float4 r0 = r[0], r1 = r[1], r2 = r[2];
+    return {f3(r0.x, r0.y, r0.z), f3(r1.x, r1.y, r1.z), f3(r2.x, r2.y, r2.z), __float_as_uint(r1.w)};
 }
 
-// FP32 copy of a posed vertex
-__device__ inline F3 vertex32(const MeshDev &m, const SlotBufs &sb, int v) { return f3(vertex(m, sb, v)); }
+// The vertices as values of unknown origin: the sweeps then contract their products
+// the same way wherever the vertices were read (another contraction moves the Sun
+// gradient, whose torque terms cancel, by 1e-7).
+__device__ __forceinline__ void pin(Tri32 &T)
+{
+    float *x = &T.A.x;
+    for (int k = 0; k < 9; k++) asm volatile("" : "+f"(x[k]));
+}
 
-// warp_scatter with FP32 lane values and FP64 accumulation
+// Add val[0..n) of the lanes holding `key` (>= 0) into row[key * n ..], for
+// every distinct key in the warp: masked butterfly sums in FP32, added in FP64 by
+// a lane a value (one FP64 instruction a key).
 template <int n>
 __device__ inline void warp_scatter32(int key, const float *val, double *row)
 {
+    const int lane = threadIdx.x & 31, c = warp_sum_value<n>(lane);
     unsigned todo = __ballot_sync(kFull, key >= 0);
     while (todo) {
         int k = __shfl_sync(kFull, key, __ffs(todo) - 1);
         bool mine = key == k;
-        float sum[n];
+        float x[n];
 #pragma unroll
-        for (int c = 0; c < n; c++) sum[c] = wsumf(mine ? val[c] : 0.0f);
-        if ((threadIdx.x & 31) == 0) {
-#pragma unroll
-            for (int c = 0; c < n; c++) row[k * n + c] += (double)sum[c];
-        }
+        for (int q = 0; q < n; q++) x[q] = mine ? val[q] : 0.0f;
+        const float sum = warp_sums<n>(x, lane);
+        if (c >= 0) row[k * n + c] += (double)sum;
         todo &= ~__ballot_sync(kFull, mine);
     }
+    __syncwarp();
 }
 
-__global__ void __launch_bounds__(kAdjThreads) k_adj_rays(AdjArgs a)
+// What bounds the kernel: FP64 instructions, at 64 cycles a warp each.  512^2 rays of a
+// 50k-triangle craft (cold caches): 70 us with FP64 sums lane by lane, constants formed in every
+// thread and vertices read in FP64 (through the vertex's part); 31 with the sums
+// above, the constants formed once a block and the FP32 records (the same bits).
+__global__ void __launch_bounds__(kAdjThreads) k_adj_rays(AdjArgs a, int G)
 {
+    pdl_enter();
     const int s = blockIdx.y;
     const SlotPose &P = a.pose[s];
     if (P.skip) return;
@@ -219,17 +209,33 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_rays(AdjArgs a)
     double *row = sh + (size_t)warp * W;
     for (int k = lane; k < W; k += 32) row[k] = 0.0;
     __syncwarp();
-    __shared__ double win[4];
-    if (threadIdx.x < 4) {
-        int vi = a.win_ids[4 * s + threadIdx.x];
-        V3 x = vertex(m, sb, vi);
-        win[threadIdx.x] = dot(threadIdx.x < 2 ? ld3(P.u) : ld3(P.v), x);
+    // the FP32 constants of the slot, formed by one warp: u, v, d, c_ref, g_F, g_T, window corner and pixel sides
+    __shared__ float cst[22];
+    if (warp == 0) {
+        int id = 0;
+        for (int c = 0; c < 4; c++) {
+            const int q = window_vertex(a, s, c, G);
+            if (lane == c) id = q;
+        }
+        const V3 x = vertex(m, sb, id);
+        const double w = dot((lane & 2) ? ld3(P.v) : ld3(P.u), x);
+        const double w0 = __shfl_sync(kFull, w, 2 * (lane & 1)), w1 = __shfl_sync(kFull, w, 2 * (lane & 1) + 1);
+        const double side = (w1 - w0) / N;
+        if (lane < 2) {
+            cst[18 + lane] = (float)w0;
+            cst[20 + lane] = (float)side;
+        }
+        if (lane < 18) {
+            const int g = lane / 3;
+            const double *src = g == 0 ? P.u : g == 1 ? P.v : g == 2 ? P.d : g == 3 ? m.c_ref
+                                : g == 4 ? a.g_force + 3 * (size_t)e : a.g_torque + 3 * (size_t)e;
+            cst[lane] = (float)src[lane % 3];
+        }
     }
     __syncthreads();
-    const F3 u = f3(ld3(P.u)), v = f3(ld3(P.v)), d0 = f3(ld3(P.d)), cref = f3(ld3(m.c_ref));
-    const F3 gF = f3(ld3(a.g_force + 3 * (size_t)e)), gT = f3(ld3(a.g_torque + 3 * (size_t)e));
-    const float umin = (float)win[0], vmin = (float)win[2];
-    const float Du = (float)((win[1] - win[0]) / N), Dv = (float)((win[3] - win[2]) / N);
+    const auto c3 = [&](int g) { return f3(cst[3 * g], cst[3 * g + 1], cst[3 * g + 2]); };
+    const F3 u = c3(0), v = c3(1), d0 = c3(2), cref = c3(3), gF = c3(4), gT = c3(5);
+    const float umin = cst[18], vmin = cst[19], Du = cst[20], Dv = cst[21];
     const size_t R = (size_t)N * N;
     F3 acc_d = f3(0, 0, 0), acc_u = f3(0, 0, 0), acc_v = f3(0, 0, 0);
     float acc_w[4] = {0, 0, 0, 0}, acc_l = 0.0f;
@@ -260,14 +266,15 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_rays(AdjArgs a)
             float w = 1.0f;
             for (int k = 0; k < nh; k++) {
                 so[k] = o; sd[k] = d; sw[k] = w;
-                int4 tv = m.tri_v4[tri[k]];
-                F3 A = vertex32(m, sb, tv.x), B = vertex32(m, sb, tv.y), C = vertex32(m, sb, tv.z);
+                Tri32 T = tri32(m, sb, tri[k]);
+                pin(T);
+                const F3 A = T.A, B = T.B, C = T.C;
                 F3 n = cross(B - A, C - A);
                 n = rsqrtf(dot(n, n)) * n;
                 float dn = dot(d, n);
                 float t = dot(n, A - o) / dn;
                 F3 x = o + t * d;
-                unsigned mp = m.tri_mat[tri[k]];
+                const unsigned mp = T.mat;
                 int mi = dn < 0.0f ? (int)(mp & 0xffffu) : (int)(mp >> 16);
                 w *= m.mat32[mi].x;
                 d = d - (2.0f * dn) * n;
@@ -284,9 +291,9 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_rays(AdjArgs a)
             if (act) {
                 const F3 o = so[k], d = sd[k];
                 const float w = sw[k];
-                const int4 tv = m.tri_v4[tri[k]];
-                const F3 A = vertex32(m, sb, tv.x), B = vertex32(m, sb, tv.y),
-                         C = vertex32(m, sb, tv.z);
+                Tri32 T = tri32(m, sb, tri[k]);
+                pin(T);
+                const F3 A = T.A, B = T.B, C = T.C;
                 const F3 e1 = B - A, e2 = C - A, mr = cross(e1, e2);
                 const float il = rsqrtf(dot(mr, mr));
                 const F3 n = il * mr;
@@ -294,7 +301,7 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_rays(AdjArgs a)
                 const F3 ao = A - o;
                 const float t = dot(n, ao) / dn;
                 const F3 x = o + t * d;
-                const unsigned mp = m.tri_mat[tri[k]];
+                const unsigned mp = T.mat;
                 const bool front = dn < 0.0f;
                 const int mi = front ? (int)(mp & 0xffffu) : (int)(mp >> 16);
                 const float2 rho = m.mat32[mi];
@@ -345,9 +352,8 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_rays(AdjArgs a)
                 mkey = mi;
                 mval[0] = rsb;
                 mval[1] = rdb;
-                const int pp = m.vert_part[tv.x];
-                if (m.part[pp].dynamic) {
-                    pkey = pp;
+                if (tri[k] >= m.n_static_tris) {  // of a dynamic part
+                    pkey = m.tri_v4[tri[k]].w >> 24;
                     const F3 G = Ab + e1b + e2b, Mm = cross(A, Ab) + cross(B, e1b) + cross(C, e2b);
                     pval[0] = G.x; pval[1] = G.y; pval[2] = G.z;
                     pval[3] = Mm.x; pval[4] = Mm.y; pval[5] = Mm.z;
@@ -373,11 +379,12 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_rays(AdjArgs a)
     }
     float fix[kAdjFixed] = {acc_d.x, acc_d.y, acc_d.z, acc_u.x, acc_u.y, acc_u.z, acc_v.x, acc_v.y, acc_v.z,
                             acc_w[0], acc_w[1], acc_w[2], acc_w[3], acc_l};
+    double fix64[kAdjFixed];
 #pragma unroll
-    for (int c = 0; c < kAdjFixed; c++) {
-        double x = wsum((double)fix[c]);
-        if (lane == 0) row[c] += x;
-    }
+    for (int c = 0; c < kAdjFixed; c++) fix64[c] = (double)fix[c];
+    const double fsum = warp_sums<kAdjFixed>(fix64, lane);
+    const int fc = warp_sum_value<kAdjFixed>(lane);
+    if (fc >= 0) row[fc] += fsum;
     __syncthreads();
     double *out = a.partials + ((size_t)s * a.nb + blockIdx.x) * W;
     for (int k = threadIdx.x; k < W; k += blockDim.x) {
@@ -394,6 +401,7 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_rays(AdjArgs a)
 // values in a row.
 __global__ void __launch_bounds__(128) k_adj_finish_sum(AdjArgs a)
 {
+    pdl_enter();
     const int s = blockIdx.y, g = blockIdx.x, G = gridDim.x, W = a.width;
     if (a.pose[s].skip) return;
     const int b0 = g * kAdjSumRun, b1 = min(b0 + kAdjSumRun, a.nb);
@@ -404,8 +412,9 @@ __global__ void __launch_bounds__(128) k_adj_finish_sum(AdjArgs a)
     }
 }
 
-__global__ void __launch_bounds__(128) k_adj_finish(AdjArgs a, int runs)
+__global__ void __launch_bounds__(128) k_adj_finish(AdjArgs a, int runs, int GW)
 {
+    pdl_enter();
     const int s = blockIdx.x;
     const SlotPose &P = a.pose[s];
     const MeshDev &m = *a.sd[s].mesh;
@@ -427,10 +436,12 @@ __global__ void __launch_bounds__(128) k_adj_finish(AdjArgs a, int runs)
         for (int b = 0; b < cnt; b++) x += src[((size_t)s * cnt + b) * W + k];
         tot[k] = x;
     }
+    __shared__ int ids[4];
+    if (threadIdx.x < 32)
+        for (int c = 0; c < 4; c++) ids[c] = window_vertex(a, s, c, GW);
     __syncthreads();
     if (threadIdx.x != 0) return;
     const int N = a.sd[s].N;
-    const int *ids = a.win_ids + 4 * s;
     V3 X[4];
     for (int c = 0; c < 4; c++) X[c] = vertex(m, sb, ids[c]);
     V3 u = ld3(P.u), v = ld3(P.v), d = ld3(P.d), sh = ld3(P.s);
@@ -534,6 +545,7 @@ __global__ void __launch_bounds__(128) k_adj_finish(AdjArgs a, int runs)
 
 __global__ void k_adj_sum(const double *g_eval, int n, int width, double *g_mat, int nm2, double *g_angle, int accumulate)
 {
+    pdl_enter();
     int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= width) return;
     double x = 0.0;
@@ -558,25 +570,24 @@ int adj_blocks(int S, size_t rays)
 
 cudaError_t launch_adjoint(const AdjArgs &a, int S, cudaStream_t st)
 {
-    // the window search over the vertices: several blocks a slot (four vertices
-    // a thread), merged in block order
-    const int G = std::max(1, std::min(kAdjWinBlocks, (a.n_verts + 4 * kAdjThreads - 1) / (4 * kAdjThreads)));
-    k_adj_window<<<dim3(G, S), kAdjThreads, 0, st>>>(a);
-    k_adj_window_merge<<<S, 32, 0, st>>>(a, G);
-    size_t smem = sizeof(double) * (size_t)kAdjWarps * a.width;
-    k_adj_rays<<<dim3(a.nb, S), kAdjThreads, smem, st>>>(a);
+    // the window search over the vertices: several blocks a slot (four vertices a thread)
+    const int G = win_blocks(a);
+    const size_t smem = sizeof(double) * (size_t)kAdjWarps * a.width;
     const int runs = a.nb > 2 * kAdjSumRun && a.partials2 ? (a.nb + kAdjSumRun - 1) / kAdjSumRun : 0;
-    if (runs > 0) k_adj_finish_sum<<<dim3(runs, S), 128, 0, st>>>(a);
-    k_adj_finish<<<S, 128, sizeof(double) * a.width, st>>>(a, runs);
-    return cudaGetLastError();
+    cudaError_t e = launch_chained(k_adj_window, dim3(G, S), dim3(kAdjThreads), 0, st, a);
+    if (e == cudaSuccess) e = launch_chained(k_adj_rays, dim3(a.nb, S), dim3(kAdjThreads), smem, st, a, G);
+    if (e == cudaSuccess && runs > 0) e = launch_chained(k_adj_finish_sum, dim3(runs, S), dim3(128), 0, st, a);
+    if (e == cudaSuccess)
+        e = launch_chained(k_adj_finish, dim3(S), dim3(128), sizeof(double) * a.width, st, a, runs, G);
+    return e;
 }
 
 cudaError_t launch_adj_sum(const double *g_eval, int n, int n_mats, int n_parts, double *g_mat, double *g_angle,
                            cudaStream_t st, bool accumulate)
 {
     int width = 2 * n_mats + n_parts;
-    k_adj_sum<<<(width + 127) / 128, 128, 0, st>>>(g_eval, n, width, g_mat, 2 * n_mats, g_angle, accumulate ? 1 : 0);
-    return cudaGetLastError();
+    return launch_chained(k_adj_sum, dim3((width + 127) / 128), dim3(128), 0, st, g_eval, n, width, g_mat, 2 * n_mats,
+                          g_angle, accumulate ? 1 : 0);
 }
 
 }  // namespace srp

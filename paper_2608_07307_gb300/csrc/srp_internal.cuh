@@ -417,6 +417,50 @@ struct PropAdj {
     double qbar[4];     // attitude quaternion cotangent, summed over the arc
 };
 
+// The warp's sums of N values a lane, by the butterfly over lane distances 16, 8, 4, 2,
+// 1: each step halves the values a lane carries (the other half goes to the partner),
+// so 6 values take 8 additions instead of 30, 14 take 15 instead of 70.  What that is
+// worth: an FP64 instruction holds the FP64 pipe for 64 cycles a warp.  The sums are
+// those of the butterfly bit for bit.  Lane l returns the sum of value
+// warp_sum_value<N>(l); of the lanes with the same value one holds it (-1 for the others).
+template <int N>
+__device__ __forceinline__ int warp_sum_value(int lane)
+{
+    constexpr int n1 = (N + 1) / 2, n2 = (n1 + 1) / 2, n3 = (n2 + 1) / 2, n4 = (n3 + 1) / 2;
+    static_assert(N >= 1 && (n4 + 1) / 2 == 1, "at most 32 values");
+    constexpr int n[5] = {N, n1, n2, n3, n4};
+    int pos = 0;
+    bool own = true;
+#pragma unroll
+    for (int s = 4; s >= 0; s--) {
+        const bool h = lane & (16 >> s);
+        const int up = pos + (n[s] + 1) / 2;
+        if (h && up < n[s]) pos = up;
+        else if (h) own = false;
+    }
+    return own ? pos : -1;
+}
+template <int N, int O, typename T>
+__device__ __forceinline__ T warp_sum_step(const T *v, int lane)
+{
+    constexpr int H = (N + 1) / 2;
+    T r[H];
+    const bool h = lane & O;
+#pragma unroll
+    for (int k = 0; k < H; k++) {
+        const T keep = h && k + H < N ? v[k + H < N ? k + H : k] : v[k];
+        const T send = k + H < N ? (h ? v[k] : v[k + H < N ? k + H : k]) : v[k];
+        r[k] = keep + __shfl_xor_sync(0xffffffffu, send, O);
+    }
+    if constexpr (O == 1) return r[0];
+    else return warp_sum_step<H, O / 2, T>(r, lane);
+}
+template <int N, typename T>
+__device__ __forceinline__ T warp_sums(const T *v, int lane)
+{
+    return warp_sum_step<N, 16, T>(v, lane);
+}
+
 // ordered-int encoding of doubles for atomicMin/Max
 __host__ __device__ inline unsigned long long dbl_to_ord(double x)
 {
@@ -481,9 +525,10 @@ struct AdjArgs {
     int panel_mode, n_mats, n_parts, eval0;
     int nb;                      // ray blocks per slot
     int width;                   // doubles per block partial (kAdjFixed + 2 n_mats + 6 n_parts)
-    int *win_ids;                // [S][4] extreme vertices: argmin u, argmax u, argmin v, argmax v
-    double *win_val;             // [S][kAdjWinBlocks][4] the window blocks' extreme projections
-    int *win_pid;                // [S][kAdjWinBlocks][4] and their vertices
+    int *win_pid;                // [S][kAdjWinBlocks][4] a window block's lowest vertex at each extreme (argmin u,
+                                 // argmax u, argmin v, argmax v), or INT_MAX
+    int records;                 // the window kernel writes the triangle records of the dynamic parts (no refit ran)
+    int n_dyn_tris;              // most dynamic triangles of the slots' meshes
     int n_verts;                 // most vertices of the slots' meshes
     double *partials;            // [S][nb][width]
     double *partials2;           // [S][ceil(nb / kAdjSumRun)][width] runs of kAdjSumRun partials summed, when nb > 2 kAdjSumRun

@@ -1312,34 +1312,6 @@ __device__ __forceinline__ void comp_merge(Comp32 &c, const Comp32 &d)
 }
 __device__ __forceinline__ float comp_value(const Comp32 &c) { return __fadd_rn(c.hi, c.lo); }
 
-__device__ inline double warp_sum(double x)
-{
-    for (int o = 16; o; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-    return x;
-}
-
-// The warp's sums of six FP64 values by warp_sum's tree, each step halving what a
-// lane carries: 8 additions instead of 30 (an FP64 instruction holds the pipe for 64
-// cycles a warp).  The sum of value sum6_value(lane) is returned in lanes 0, 4, 8, 16, 20, 24.
-__device__ __forceinline__ int sum6_value(int lane)
-{
-    return (lane & 16 ? 3 : 0) + (lane & 4 ? 1 : lane & 8 ? 2 : 0);
-}
-__device__ __forceinline__ bool sum6_holds(int lane) { return (lane & 3) == 0 && (lane & 12) != 12; }
-__device__ __forceinline__ double warp_sum6(const double *v, int lane)
-{
-    const auto other = [](double x, int o) { return __shfl_xor_sync(0xffffffffu, x, o); };
-    const bool h16 = lane & 16, h8 = lane & 8, h4 = lane & 4;
-    double a[3];
-    for (int k = 0; k < 3; k++) a[k] = (h16 ? v[3 + k] : v[k]) + other(h16 ? v[k] : v[3 + k], 16);
-    const double b0 = (h8 ? a[2] : a[0]) + other(h8 ? a[0] : a[2], 8);
-    const double b1 = a[1] + other(a[1], 8);
-    double c = (h4 ? b1 : b0) + other(h4 ? b0 : b1, 4);
-    c += other(c, 2);
-    c += other(c, 1);
-    return c;
-}
-
 // Slot of flattened trace block g: the last slot whose first block is <= g.
 __device__ __forceinline__ int slot_of_block(const SlotDesc *sd, int S, int g)
 {
@@ -2909,10 +2881,9 @@ __global__ void __launch_bounds__(kLaneStride, 4) k_diffuse(TraceArgs a)
     }
     // block sum in a fixed order: warps by shuffles, then the four warps in turn
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int k = 0; k < 6; k++) {
-        const double x = warp_sum(acc[k]);
-        if (lane == 0) red[w][k] = x;
-    }
+    const double sum = warp_sums<6>(acc, lane);
+    const int kv = warp_sum_value<6>(lane);
+    if (kv >= 0) red[w][kv] = sum;
     __syncthreads();
     if (threadIdx.x < 6) {
         const int k = threadIdx.x;
@@ -2995,8 +2966,9 @@ __global__ void __launch_bounds__(256) k_reduce1(TraceArgs a, int eval0, double 
     __shared__ Comp32 r32[6][256];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (mode == 0) {
-        const double x = warp_sum6(f, lane);
-        if (sum6_holds(lane)) rf[sum6_value(lane)][w] = x;
+        const double x = warp_sums<6>(f, lane);
+        const int k = warp_sum_value<6>(lane);
+        if (k >= 0) rf[k][w] = x;
     } else {
         for (int k = 0; k < 6; k++) r32[k][threadIdx.x] = f32[k];
     }
@@ -3062,8 +3034,9 @@ __device__ void final_reduce(const TraceArgs &a, int s, int eval0, double *force
     if (w < kRed1 / 32) {
         double v[6];
         for (int k = 0; k < 6; k++) v[k] = first(threadIdx.x, k);
-        const double x = warp_sum6(v, lane);
-        if (sum6_holds(lane)) red2[sum6_value(lane)][w] = x;
+        const double x = warp_sums<6>(v, lane);
+        const int k = warp_sum_value<6>(lane);
+        if (k >= 0) red2[k][w] = x;
     }
     if (w == nw - 1) {
         const SlotPose &P = a.pose[s];
