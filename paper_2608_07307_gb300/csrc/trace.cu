@@ -2342,6 +2342,27 @@ __device__ void tri_v64(const TraceCtx &B, int p, int tl, double *v)
     }
 }
 
+// FP64 signs and comparisons by their bits (an FP64 comparison holds the FP64 pipe
+// like an addition: 64 cycles a warp): x < 0 and x > 0 of a number that is not NaN,
+// a > b where b is not negative.
+__device__ __forceinline__ bool neg64(double x)
+{
+    return __double2hiint(x) < 0 && ((__double2hiint(x) & 0x7fffffff) | __double2loint(x)) != 0;
+}
+__device__ __forceinline__ bool pos64(double x) { return __double_as_longlong(x) > 0; }
+__device__ __forceinline__ bool above64(double a, double b) { return __double_as_longlong(a) > __double_as_longlong(b); }
+// the edge functions have both signs: the line misses the triangle
+__device__ __forceinline__ bool missed64(double U, double V, double W)
+{
+    return (neg64(U) || neg64(V) || neg64(W)) && (pos64(U) || pos64(V) || pos64(W));
+}
+__device__ __forceinline__ bool zero64(double x) { return ((__double2hiint(x) & 0x7fffffff) | __double2loint(x)) == 0; }
+// the nearer of two hits above tlo >= 0: equal distances go to the lowest original id
+__device__ __forceinline__ bool nearer64(double t, int orig, double tlo, double bt, int bo)
+{
+    return above64(t, tlo) && (above64(bt, t) || (__double_as_longlong(t) == __double_as_longlong(bt) && orig < bo));
+}
+
 // FP64 watertight edge functions and scaled depth of triangle v against ray r.
 __device__ __forceinline__ void wt64(const Ray64 &r, const double *v, double &U, double &V, double &W, double &det,
                                      double &T)
@@ -2425,10 +2446,9 @@ __device__ __noinline__ Best32 resolve64(const TraceCtx &B, int N, int i, int j,
             tri_v64(B, p, tl, v);
             wt64(r, v, U, V, W, det, T);
         }
-        bool out = (U < 0.0 || V < 0.0 || W < 0.0) && (U > 0.0 || V > 0.0 || W > 0.0);
-        if (out || det == 0.0) continue;
+        if (missed64(U, V, W) || zero64(det)) continue;
         double t = T / det;
-        if (t > tlo && (t < bt || (t == bt && orig < bo))) {
+        if (nearer64(t, orig, tlo, bt, bo)) {
             bt = t; bp = p; btl = tl; bo = orig; bU = det; bV = V; bW = W;
         }
     }
@@ -2505,24 +2525,11 @@ __device__ void nearest64(const TraceCtx &B, const Ray64 &r, double tlo, int ski
                 if (orig != skip && !outside32(q, fa, fb, fc, dq)) {
                     double v[9];
                     tri_v64(B, p, tl, v);
-                    double A[3], Bv[3], C[3];
-                    for (int k = 0; k < 3; k++) { A[k] = v[k] - r.o[k]; Bv[k] = v[3 + k] - r.o[k]; C[k] = v[6 + k] - r.o[k]; }
-                    double Akz = pickd(A[0], A[1], A[2], r.kz), Bkz = pickd(Bv[0], Bv[1], Bv[2], r.kz),
-                           Ckz = pickd(C[0], C[1], C[2], r.kz);
-                    double Ax = pickd(A[0], A[1], A[2], r.kx) - r.Sx * Akz, Ay = pickd(A[0], A[1], A[2], r.ky) - r.Sy * Akz;
-                    double Bx = pickd(Bv[0], Bv[1], Bv[2], r.kx) - r.Sx * Bkz, By = pickd(Bv[0], Bv[1], Bv[2], r.ky) - r.Sy * Bkz;
-                    double Cx = pickd(C[0], C[1], C[2], r.kx) - r.Sx * Ckz, Cy = pickd(C[0], C[1], C[2], r.ky) - r.Sy * Ckz;
-                    double U = __dsub_rn(__dmul_rn(Cx, By), __dmul_rn(Cy, Bx));
-                    double V = __dsub_rn(__dmul_rn(Ax, Cy), __dmul_rn(Ay, Cx));
-                    double W = __dsub_rn(__dmul_rn(Bx, Ay), __dmul_rn(By, Ax));
-                    bool out = (U < 0.0 || V < 0.0 || W < 0.0) && (U > 0.0 || V > 0.0 || W > 0.0);
-                    double det = U + V + W;
-                    if (!out && det != 0.0) {
-                        double T = U * (r.Sz * Akz) + V * (r.Sz * Bkz) + W * (r.Sz * Ckz);
-                        double t = T / det;
-                        if (t > tlo && (t < bt || (t == bt && orig < borig))) {
-                            bt = t; bpart = p; btl = tl; borig = orig;
-                        }
+                    double U, V, W, det, T;
+                    wt64(r, v, U, V, W, det, T);
+                    if (!missed64(U, V, W) && !zero64(det)) {
+                        const double t = T / det;
+                        if (nearer64(t, orig, tlo, bt, borig)) { bt = t; bpart = p; btl = tl; borig = orig; }
                     }
                 }
             }
@@ -2532,8 +2539,112 @@ __device__ void nearest64(const TraceCtx &B, const Ray64 &r, double tlo, int ski
     }
 }
 
+// nearest64 of one ray by a warp (every lane calls it with the same ray): lanes take
+// the nodes and triangles of one list, so a step's loads and a triangle's FP64 test
+// cover up to 32 of them.  The result is the same: the least (t, original id) of the
+// triangles not certainly missed or beyond it, in whatever order they are met.
+constexpr int kWalk64 = 64;  // list entries (part, reference) beside the depth-first reserve
+struct Walk64 {
+    int2 e[kWalk64 + kStack];
+};
+__device__ __noinline__ void nearest64_warp(const TraceCtx &B, Walk64 &S, const Ray64 &r, double tlo, int skip,
+                                            double &bt, int &bpart, int &btl, int &borig, int &flags)
+{
+    constexpr unsigned kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const unsigned below = (1u << lane) - 1u;
+    bt = INFINITY;
+    bpart = -1; btl = -1; borig = 0x7fffffff;
+    Ray32 q;
+    for (int k = 0; k < 3; k++) { q.o[k] = (float)r.o[k]; q.d[k] = (float)r.d[k]; }
+    ray_setup(q);
+    const float slack = 4.0f * B.pad, tn = (float)tlo - slack;
+    const float omax = fmaxf(fmaxf(fabsf(q.o[0]), fabsf(q.o[1])), fabsf(q.o[2]));
+    const float dq = 2.0f * kU * (omax + B.R);
+    // the parts whose box the ray enters, a lane each
+    int n, limit;
+    {
+        bool in = false;
+        int lim = 0;
+        if (lane < B.n_parts) {
+            const PartView &pv = B.part[lane];
+            in = box_enter(pv.box[0], pv.box[3], pv.box[1], pv.box[4], pv.box[2], pv.box[5], q.inv, q.oi, tn, INFINITY) !=
+                 INFINITY;
+            lim = in ? pv.limit : 0;
+        }
+        const unsigned m = __ballot_sync(kAll, in);
+        if (in) S.e[__popc(m & below)] = make_int2(lane, B.part[lane].root);
+        n = __popc(m);
+        limit = __reduce_add_sync(kAll, lim);
+    }
+    __syncwarp();
+    while (n > 0) {
+        // as many as their children have room for; one at a time at the end of the room,
+        // which is then a depth-first walk and stays within the reserve
+        const int m = min(min(n, 32), max(1, (kWalk64 - n) / 3));
+        if ((limit -= m) < 0) { flags |= kFlagStack; break; }
+        const bool mine = lane < m;
+        int2 e = make_int2(0, 0);
+        if (mine) e = S.e[n - 1 - lane];
+        n -= m;
+        __syncwarp();
+        int4 c = make_int4(0, 0, 0, 0);
+        bool in[4] = {false, false, false, false};
+        bool test = false;
+        int orig = 0x7fffffff;
+        const float thi = (float)bt + slack;
+        if (mine && e.y >= 0) {
+            const float4 *nd = B.part[e.x].node + (size_t)e.y * kNode4;
+            const int ox = q.code & 1, oy = (q.code >> 1) & 1, oz = (q.code >> 2) & 1;
+            const float4 nx = __ldg(nd + ox), fx = __ldg(nd + 1 - ox), ny = __ldg(nd + 2 + oy), fy = __ldg(nd + 3 - oy),
+                         nz = __ldg(nd + 4 + oz), fz = __ldg(nd + 5 - oz);
+            c = __ldg(reinterpret_cast<const int4 *>(nd + 6));
+            in[0] = box_enter_nf(nx.x, fx.x, ny.x, fy.x, nz.x, fz.x, q.inv, q.oi, tn, thi) != INFINITY;
+            in[1] = box_enter_nf(nx.y, fx.y, ny.y, fy.y, nz.y, fz.y, q.inv, q.oi, tn, thi) != INFINITY;
+            in[2] = box_enter_nf(nx.z, fx.z, ny.z, fy.z, nz.z, fz.z, q.inv, q.oi, tn, thi) != INFINITY;
+            in[3] = box_enter_nf(nx.w, fx.w, ny.w, fy.w, nz.w, fz.w, q.inv, q.oi, tn, thi) != INFINITY;
+        } else if (mine) {
+            const float4 *tr = B.part[e.x].tri + (size_t)(~e.y) * 3;
+            const float4 fa = __ldg(tr), fb = __ldg(tr + 1), fc = __ldg(tr + 2);
+            orig = __float_as_int(fa.w);
+            test = orig != skip && !outside32(q, fa, fb, fc, dq);
+        }
+        const int ck[4] = {c.x, c.y, c.z, c.w};
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            const unsigned mk = __ballot_sync(kAll, in[k]);
+            if (in[k]) S.e[n + __popc(mk & below)] = make_int2(e.x, ck[k]);
+            n += __popc(mk);
+        }
+        if (__any_sync(kAll, test)) {
+            double t = INFINITY;
+            bool hit = false;
+            if (test) {
+                double v[9], U, V, W, det, T;
+                tri_v64(B, e.x, ~e.y, v);
+                wt64(r, v, U, V, W, det, T);
+                if (!missed64(U, V, W) && !zero64(det)) {
+                    t = T / det;
+                    hit = nearer64(t, orig, tlo, bt, borig);
+                }
+            }
+            unsigned todo = __ballot_sync(kAll, hit);
+            while (todo) {  // (few: hits nearer than what the earlier steps left)
+                const int l = __ffs(todo) - 1;
+                todo &= todo - 1u;
+                const double tl = __shfl_sync(kAll, t, l);
+                const int ol = __shfl_sync(kAll, orig, l), pl = __shfl_sync(kAll, e.x, l), rl = __shfl_sync(kAll, e.y, l);
+                if (nearer64(tl, ol, tlo, bt, borig)) { bt = tl; bpart = pl; btl = ~rl; borig = ol; }
+            }
+        }
+        __syncwarp();
+    }
+}
+
 // Re-trace of one handed-off ray, FP64 from the pixel definition; adds to acc.
-__device__ void refine_ray(const TraceCtx &B, const TraceArgs &a, int s, int ray, double *acc, int &flags)
+// (walk: by the whole warp, every lane with the same ray; null: by one lane)
+__device__ __noinline__ void refine_ray(const TraceCtx &B, const TraceArgs &a, int s, int ray, Walk64 *walk, double *acc,
+                                        int &flags)
 {
     const int N = a.sd[s].N, nseg = a.sd[s].nseg;
     int i = ray / N, j = ray % N;
@@ -2551,7 +2662,8 @@ __device__ void refine_ray(const TraceCtx &B, const TraceArgs &a, int s, int ray
         double t;
         int hpart, htl, horig;
         nseg_done++;
-        nearest64(B, r, seg == 0 ? 0.0 : B.eps, skip, t, hpart, htl, horig, flags);
+        if (walk) nearest64_warp(B, *walk, r, seg == 0 ? 0.0 : B.eps, skip, t, hpart, htl, horig, flags);
+        else nearest64(B, r, seg == 0 ? 0.0 : B.eps, skip, t, hpart, htl, horig, flags);
         if (hpart < 0) break;
         if (hp) hp[seg] = horig;
         acc[8 + seg] += 1.0;
@@ -2651,10 +2763,9 @@ __device__ void settle64(const TraceCtx &B, const Ray64 &r, double tlo, int skip
         double v[9], U, V, W, det, T;
         tri_v64(B, p, tl, v);
         wt64(r, v, U, V, W, det, T);
-        const bool out = (U < 0.0 || V < 0.0 || W < 0.0) && (U > 0.0 || V > 0.0 || W > 0.0);
-        if (out || det == 0.0) continue;
+        if (missed64(U, V, W) || zero64(det)) continue;
         const double t = T / det;
-        if (t > tlo && (t < bt || (t == bt && orig < bo))) { bt = t; bp = p; btl = tl; bo = orig; }
+        if (nearer64(t, orig, tlo, bt, bo)) { bt = t; bp = p; btl = tl; bo = orig; }
     }
 }
 
@@ -2900,7 +3011,75 @@ __global__ void __launch_bounds__(kLaneStride, 4) k_diffuse(TraceArgs a)
 __device__ void final_reduce(const TraceArgs &a, int s, int eval0, double *force, double *torque, int *err_flags,
                              unsigned long long *stats_accum, bool cg);
 
-__global__ void __launch_bounds__(256) k_reduce1(TraceArgs a, int eval0, double *force, double *torque,
+// Re-traced rays of a block that its warps take one by one (nearest64_warp); with more, a lane
+// a ray.  A warp takes 40-60 us a ray and a block has eight warps; a lane takes 100-350 us, but
+// up to 32 of them run at once: the two meet near four rays a warp.
+constexpr int kWarpRays = 32;
+// Warps of a first-level block, resident blocks: 32 box-wing evaluations a launch 39 us at two
+// blocks an SM (128 registers), 32.6 at four (the re-trace spills, rarely run), 31.6 at five.
+constexpr int kRedWarps = 8, kRedBlocksPerSM = 4;
+
+struct RefineShared {
+    int n[kRedWarps], first[32 * kRedWarps];
+    double sum[kRedWarps][kPart];
+    Walk64 walk[kRedWarps];
+};
+
+// The re-trace of the rays that tiles [t0, t1) of slot s handed off, summed by the
+// thread that owns the tile into its acc.  (Out of line: rare, and its registers are not
+// the reduction's.)  200k triangles, 1024^2, two bounces, eight evaluations: 366 -> 131 us
+// where rays overflow, a warp a ray against a lane a ray.
+__device__ __noinline__ void refine_block(const TraceCtx &B, const TraceArgs &a, int s, int t0, int t1, size_t base,
+                                          RefineShared &S, double *acc, int &flags)
+{
+    // the block's rays in the order of its threads: own of them from first
+    int own = 0;
+    for (int t = t0 + (int)threadIdx.x; t < t1; t += blockDim.x) own += a.amb_count[base + t];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int first = own;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(0xffffffffu, first, o);
+        if (lane >= o) first += x;
+    }
+    if (lane == 31) S.n[w] = first;
+    __syncthreads();
+    int total = 0;
+    for (int q = 0; q < kRedWarps; q++) {
+        if (q == w) first += total - own;
+        total += S.n[q];
+    }
+    if (total <= kWarpRays) {
+        // few: a warp a ray, added by the owners in their order
+        S.first[threadIdx.x] = first;
+        for (int r0 = 0; r0 < total; r0 += kRedWarps) {
+            __syncthreads();
+            const int ray = r0 + w;
+            if (ray < total) {
+                int o = 0;  // the last thread that starts at or before it
+                for (int h = kRedWarps * 16; h; h >>= 1)
+                    if (S.first[o + h] <= ray) o += h;
+                int q = ray - S.first[o], t = t0 + o;
+                for (int c; q >= (c = a.amb_count[base + t]); t += blockDim.x) q -= c;
+                double x[kPart];
+                for (int k = 0; k < kPart; k++) x[k] = 0.0;
+                refine_ray(B, a, s, a.amb_list[(base + t) * kTileRays + q], &S.walk[w], x, flags);
+                if (lane == 0)
+                    for (int k = 0; k < kPart; k++) S.sum[w][k] = x[k];
+            }
+            __syncthreads();
+            for (int q = 0; q < kRedWarps; q++)
+                if (r0 + q >= first && r0 + q < first + own)
+                    for (int k = 0; k < kPart; k++) acc[k] += S.sum[q][k];
+        }
+    } else {
+        for (int t = t0 + (int)threadIdx.x; t < t1; t += blockDim.x) {
+            const int n = a.amb_count[base + t];
+            for (int q = 0; q < n; q++) refine_ray(B, a, s, a.amb_list[(base + t) * kTileRays + q], nullptr, acc, flags);
+        }
+    }
+}
+
+__global__ void __launch_bounds__(32 * kRedWarps, kRedBlocksPerSM) k_reduce1(TraceArgs a, int eval0, double *force, double *torque,
                                                  int *err_flags, unsigned long long *stats_accum, int fuse)
 {
     pdl_enter();
@@ -2938,6 +3117,10 @@ __global__ void __launch_bounds__(256) k_reduce1(TraceArgs a, int eval0, double 
     }
     __shared__ TraceCtx B;
     __shared__ int blk_flags;
+    __shared__ union {  // (40 KB side by side made a launch of eight evaluations 2 us slower)
+        RefineShared re;
+        Comp32 r32[6][32 * kRedWarps];
+    } sh;
     if (__syncthreads_or(mine)) {
         if (threadIdx.x == 0) blk_flags = 0;
         load_ctx(B, a, s);
@@ -2945,10 +3128,7 @@ __global__ void __launch_bounds__(256) k_reduce1(TraceArgs a, int eval0, double 
         int flags = 0;
         double acc[kPart];
         for (int k = 0; k < kPart; k++) acc[k] = 0.0;
-        for (int t = t0 + (int)threadIdx.x; t < t1; t += blockDim.x) {
-            const int n = a.amb_count[base + t];
-            for (int q = 0; q < n; q++) refine_ray(B, a, s, a.amb_list[(base + t) * kTileRays + q], acc, flags);
-        }
+        refine_block(B, a, s, t0, t1, base, sh.re, acc, flags);
         for (int k = 0; k < 6; k++) {
             if (mode == 0) f[k] += acc[k];
             else if (mode == 1) comp_add(f32[k], (float)acc[k]);
@@ -2963,14 +3143,13 @@ __global__ void __launch_bounds__(256) k_reduce1(TraceArgs a, int eval0, double 
     // modes' sums, threads in turn by one thread), integers for counts
     __shared__ double rf[6][8];
     __shared__ unsigned long long rc[kCnt][8];
-    __shared__ Comp32 r32[6][256];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (mode == 0) {
         const double x = warp_sums<6>(f, lane);
         const int k = warp_sum_value<6>(lane);
         if (k >= 0) rf[k][w] = x;
     } else {
-        for (int k = 0; k < 6; k++) r32[k][threadIdx.x] = f32[k];
+        for (int k = 0; k < 6; k++) sh.r32[k][threadIdx.x] = f32[k];
     }
     for (int k = 0; k < kCnt; k++) {
         // only the live counts (kc is uniform over the launch)
@@ -2988,8 +3167,8 @@ __global__ void __launch_bounds__(256) k_reduce1(TraceArgs a, int eval0, double 
         } else {
             Comp32 x{0.0f, 0.0f};
             for (int q = 0; q < (int)blockDim.x; q++) {
-                if (mode == 1) comp_merge(x, r32[threadIdx.x][q]);
-                else x.hi = __fadd_rn(x.hi, r32[threadIdx.x][q].hi);
+                if (mode == 1) comp_merge(x, sh.r32[threadIdx.x][q]);
+                else x.hi = __fadd_rn(x.hi, sh.r32[threadIdx.x][q].hi);
             }
             out[threadIdx.x] = (double)comp_value(x);  // an FP32 value, exact in FP64
         }
@@ -3306,7 +3485,7 @@ cudaError_t launch_reduce(const TraceArgs &a, int S, int eval0, double *force, d
 {
     // without diffuse rays the last first-level block of a slot does the second level
     const int fuse = (a.n_diffuse <= 0 && a.red_ticket) ? 1 : 0;
-    cudaError_t e = launch_chained(k_reduce1, dim3(kRed1, S), dim3(256), 0, st, a, eval0, force, torque, err_flags,
+    cudaError_t e = launch_chained(k_reduce1, dim3(kRed1, S), dim3(32 * kRedWarps), 0, st, a, eval0, force, torque, err_flags,
                                    stats_accum, fuse);
     if (e != cudaSuccess || fuse) return e;
     // diffuse secondaries after the FP64 re-trace (which records the hits of the rays it takes)
