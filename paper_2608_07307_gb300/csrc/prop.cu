@@ -92,18 +92,6 @@ __device__ void sun_pos(double mjd_tt, double *r)
     r[2] = rr * sl * se;
 }
 
-// LVLH frame at y: columns x_b = y_b x z_b, y_b = -orbit normal, z_b = nadir
-__device__ void lvlh_matrix(const double *y, double *L)
-{
-    const double irn = -1.0 / sqrt(y[0] * y[0] + y[1] * y[1] + y[2] * y[2]);
-    double h[3] = {y[1] * y[5] - y[2] * y[4], y[2] * y[3] - y[0] * y[5], y[0] * y[4] - y[1] * y[3]};
-    const double ihn = -1.0 / sqrt(h[0] * h[0] + h[1] * h[1] + h[2] * h[2]);
-    double zb[3] = {y[0] * irn, y[1] * irn, y[2] * irn};
-    double yb[3] = {h[0] * ihn, h[1] * ihn, h[2] * ihn};
-    double xb[3] = {yb[1] * zb[2] - yb[2] * zb[1], yb[2] * zb[0] - yb[0] * zb[2], yb[0] * zb[1] - yb[1] * zb[0]};
-    for (int k = 0; k < 3; k++) { L[3 * k] = xb[k]; L[3 * k + 1] = yb[k]; L[3 * k + 2] = zb[k]; }
-}
-
 // cfg (null: P's values for every trajectory): [n][8] central, attitude, q[4], mass, unused
 __global__ void k_prop_init(PropState *S, int n, const double *y0, const double *t01, PropDev P, const double *cfg,
                             int *n_done)
@@ -593,138 +581,170 @@ __global__ void k_prop_record(const PropState *S, int n, const double *sun, cons
     rec_dist[i] = dist[i];
 }
 
-// kbar of this stage, and the cotangent of the body-frame SRP force
-__global__ void k_adj_prop_in(int n, PropDev P, int stage, const StageRec *rec, PropAdj *A, double *g_force)
+// kbar of this stage, and the cotangent of the body-frame SRP force; a warp per
+// trajectory, a component a lane
+__global__ void __launch_bounds__(32) k_adj_prop_in(int n, PropDev P, int stage, const StageRec *rec, PropAdj *A,
+                                                    double *g_force)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+    pdl_enter();
+    const int i = blockIdx.x, lane = threadIdx.x;
     const StageRec &r = rec[i];
     PropAdj &X = A[i];
     const double h = r.hs;
     const double anext = stage == 2 ? 1.0 : 0.5;  // a_{stage+1, stage}
-    for (int k = 0; k < 6; k++)
-        X.kbar[k] = h * cB4[stage] * X.lam[k] + (stage < 3 ? h * anext * X.ybar[stage + 1][k] : 0.0);
-    const double *ab = X.kbar + 3;
-    for (int k = 0; k < 3; k++)
-        g_force[3 * i + k] = r.lit ? (r.R[k] * ab[0] + r.R[3 + k] * ab[1] + r.R[6 + k] * ab[2]) / P.mass : 0.0;
+    const int k = lane < 6 ? lane : 0, c3 = lane % 3;
+    const double R0 = r.R[c3], R1 = r.R[3 + c3], R2 = r.R[6 + c3];
+    const double kb = h * cB4[stage] * X.lam[k] + (stage < 3 ? h * anext * X.ybar[stage + 1][k] : 0.0);
+    if (lane < 6) X.kbar[k] = kb;
+    const double a0 = shfl(kb, 3), a1 = shfl(kb, 4), a2 = shfl(kb, 5);
+    if (lane < 3) g_force[3 * i + lane] = r.lit ? (R0 * a0 + R1 * a1 + R2 * a2) / P.mass : 0.0;
 }
 
-// (df/dy)^T kbar at this stage: gravity, SRP through the Sun direction,
-// distance and attitude; attitude quaternion cotangent
-__global__ void k_adj_prop_out(int n, PropDev P, int stage, const StageRec *rec, PropAdj *A, const double *g_sun,
-                               const double *g_dist)
+// (df/dy)^T kbar at this stage: gravity, SRP through the Sun direction, distance
+// and attitude; attitude quaternion cotangent.  Four warps a trajectory on the SM's
+// four FP64 pipes (64 cycles an instruction and warp): central body and J2, the Sun's
+// force and direction, the quaternion, the LVLH frame and the third body; components,
+// matrix elements and quotients a lane each.  (One thread: 649 instructions in a row, 26 us.)
+__global__ void __launch_bounds__(128) k_adj_prop_out(int n, PropDev P, int stage, const StageRec *rec, PropAdj *A,
+                                                      const double *g_sun, const double *g_dist)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+    pdl_enter();
+    const int i = blockIdx.x, w = threadIdx.x >> 5, lane = threadIdx.x & 31, c3 = lane % 3;
+    const int k1 = c3 == 2 ? 0 : c3 + 1, k2 = c3 == 0 ? 2 : c3 - 1;
+    const int l9 = lane < 9 ? lane : 0, a = l9 / 3, b = l9 % 3;
     const StageRec &r = rec[i];
     PropAdj &X = A[i];
-    const double *y = r.ys, *ab = X.kbar + 3;
-    double rb[3] = {0, 0, 0}, vb[3] = {X.kbar[0], X.kbar[1], X.kbar[2]};  // x' = v
-    // central body: J = -mu (I / r^3 - 3 r r^T / r^5), symmetric
-    {
-        double r2 = y[0] * y[0] + y[1] * y[1] + y[2] * y[2], rn = sqrt(r2);
-        double mu = P.central == 1 ? kMuSun : kMuEarth;
-        double ra = y[0] * ab[0] + y[1] * ab[1] + y[2] * ab[2];
-        // one reciprocal instead of a division per term (GB300's FP64 divisions are long chains)
-        const double ir3 = 1.0 / (r2 * rn), ir5 = ir3 / r2;
-        for (int k = 0; k < 3; k++) rb[k] += -mu * (ab[k] * ir3 - 3.0 * y[k] * ra * ir5);
+    __shared__ double s_y[6], s_ab[3], s_rs[3], s_gs[3];
+    __shared__ double s_grav[3], s_third[3], s_wb[3], s_Rb[9], s_Q[9], s_Qb[9], s_L[9], s_Lb[9], s_in[2], s_rv[6];
+    if (threadIdx.x < 6) s_y[threadIdx.x] = r.ys[threadIdx.x];
+    if (w == 1 && lane < 3) {
+        s_ab[lane] = X.kbar[3 + lane];
+        s_rs[lane] = r.rsun[lane];
+        s_gs[lane] = r.lit ? g_sun[3 * i + lane] : 0.0;
     }
-    if (P.central == 0 && P.j2) {
-        double r2 = y[0] * y[0] + y[1] * y[1] + y[2] * y[2];
-        const double ir2 = 1.0 / r2;
-        double z2 = y[2] * y[2] * ir2;
-        double f = -1.5 * kJ2 * kMuEarth * kREarth * kREarth / (r2 * r2 * sqrt(r2));
-        double g[3] = {y[0] * (1.0 - 5.0 * z2), y[1] * (1.0 - 5.0 * z2), y[2] * (3.0 - 5.0 * z2)};
-        double fb = ab[0] * g[0] + ab[1] * g[1] + ab[2] * g[2];
-        rb[0] += f * ab[0] * (1.0 - 5.0 * z2);
-        rb[1] += f * ab[1] * (1.0 - 5.0 * z2);
-        rb[2] += f * ab[2] * (3.0 - 5.0 * z2);
-        double z2b = -5.0 * f * (ab[0] * y[0] + ab[1] * y[1] + ab[2] * y[2]);
-        rb[2] += z2b * 2.0 * y[2] * ir2;
-        double r2b = -z2b * y[2] * y[2] * (ir2 * ir2) + fb * (-2.5) * f * ir2;
-        for (int k = 0; k < 3; k++) rb[k] += 2.0 * r2b * y[k];
-    }
-    if (P.central == 0 && P.sun3) {
-        double d[3] = {r.rsun[0] - y[0], r.rsun[1] - y[1], r.rsun[2] - y[2]};
-        double d2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2], dn = sqrt(d2);
-        double da = d[0] * ab[0] + d[1] * ab[1] + d[2] * ab[2];
-        const double id3 = 1.0 / (d2 * dn), id5 = id3 / d2;
-        for (int k = 0; k < 3; k++) rb[k] += -kMuSun * (ab[k] * id3 - 3.0 * d[k] * da * id5);
-    }
-    if (r.lit) {
+    const bool lit = r.lit, lvlh = P.attitude != 1;  // uniform over the block
+    __syncthreads();
+    const double *y = s_y, *ab = s_ab;
+    double qn = 1.0, qk = 0.0;  // warp 2: the quaternion's norm, its normalised components in lanes 0-3
+    if (w == 0) {
+        // central body: J = -mu (I / r^3 - 3 r r^T / r^5), symmetric
+        const double r2 = y[0] * y[0] + y[1] * y[1] + y[2] * y[2], rn = sqrt(r2);
+        const double mu = P.central == 1 ? kMuSun : kMuEarth;
+        const double ra = y[0] * ab[0] + y[1] * ab[1] + y[2] * ab[2];
+        const double kJ = -1.5 * kJ2 * kMuEarth * kREarth * kREarth;
+        const double q = (lane == 2 ? kJ : 1.0) / (lane == 2 ? r2 * r2 * rn : lane == 1 ? r2 : r2 * rn);
+        const double ir3 = shfl(q, 0), ir2 = shfl(q, 1), f = shfl(q, 2);
+        const double ir5 = ir3 / r2;
+        double x = -mu * (ab[c3] * ir3 - 3.0 * y[c3] * ra * ir5);
+        if (P.central == 0 && P.j2) {
+            const double z2 = y[2] * y[2] * ir2;
+            const double m = (c3 == 2 ? 3.0 : 1.0) - 5.0 * z2;
+            const double g = y[c3] * m;
+            const double fb = ab[0] * shfl(g, 0) + ab[1] * shfl(g, 1) + ab[2] * shfl(g, 2);
+            const double z2b = -5.0 * f * ra;
+            const double r2b = -z2b * y[2] * y[2] * (ir2 * ir2) + fb * (-2.5) * f * ir2;
+            x += f * ab[c3] * m;
+            x += c3 == 2 ? z2b * 2.0 * y[2] * ir2 : 0.0;
+            x += 2.0 * r2b * y[c3];
+        }
+        if (lane < 3) s_grav[lane] = x;
+    } else if (w == 1 && lit) {
         // a_SRP = R F / m, s_body = R^T s_hat, s_hat = w / |w|, w = r_sun - r, dist = |w| / AU
-        const double *R = r.R, *gs = g_sun + 3 * i;
-        double Rb[9];
-        const double im = 1.0 / P.mass;
-        for (int a = 0; a < 3; a++)
-            for (int b = 0; b < 3; b++) Rb[3 * a + b] = ab[a] * r.F[b] * im;
-        double w[3] = {r.rsun[0] - y[0], r.rsun[1] - y[1], r.rsun[2] - y[2]};
-        double wn = sqrt(w[0] * w[0] + w[1] * w[1] + w[2] * w[2]);
-        const double iwn = 1.0 / wn;
-        double sh[3] = {w[0] * iwn, w[1] * iwn, w[2] * iwn};
-        double shb[3];
-        for (int a = 0; a < 3; a++) {
-            shb[a] = R[3 * a] * gs[0] + R[3 * a + 1] * gs[1] + R[3 * a + 2] * gs[2];
-            for (int b = 0; b < 3; b++) Rb[3 * a + b] += sh[a] * gs[b];
+        const double wv = s_rs[c3] - y[c3];
+        const double w0 = shfl(wv, 0), w1 = shfl(wv, 1), w2 = shfl(wv, 2);
+        const double wn = sqrt(w0 * w0 + w1 * w1 + w2 * w2);
+        const double q = 1.0 / (lane == 1 ? P.mass : wn);
+        const double iwn = shfl(q, 0), im = shfl(q, 1);
+        const double sc = wv * iwn;
+        const double sh0 = shfl(sc, 0), sh1 = shfl(sc, 1), sh2 = shfl(sc, 2);
+        const double *R = r.R;
+        const double shb = R[3 * c3] * s_gs[0] + R[3 * c3 + 1] * s_gs[1] + R[3 * c3 + 2] * s_gs[2];
+        const double sd = shfl(shb, 0) * sh0 + shfl(shb, 1) * sh1 + shfl(shb, 2) * sh2;
+        const double wb = (shb - sd * sc) * iwn + g_dist[i] * sc * (1.0 / kAU);
+        if (lane < 3) s_wb[lane] = wb;
+        const double Rb = ab[a] * r.F[b] * im + (a == 0 ? sh0 : a == 1 ? sh1 : sh2) * s_gs[b];
+        if (lane < 9) s_Rb[lane] = Rb;
+    } else if (w == 2 && lit) {
+        // the normalised quaternion and its rotation
+        qn = sqrt(P.q[0] * P.q[0] + P.q[1] * P.q[1] + P.q[2] * P.q[2] + P.q[3] * P.q[3]);
+        qk = P.q[lane & 3] / qn;
+        const double qw = shfl(qk, 0), qx = shfl(qk, 1), qy = shfl(qk, 2), qz = shfl(qk, 3);
+        // diagonal 1 - 2 (p p + q q), off it 2 (p q -+ w r)
+        const double v[3] = {qx, qy, qz};
+        const int o = a == b ? 0 : 3 - a - b;
+        const double p1 = a == b ? v[a == 0 ? 1 : 0] : v[a], q1 = a == b ? p1 : v[b];
+        const double p2 = a == b ? v[a == 2 ? 1 : 2] : ((b - a + 3) % 3 == 1 ? -qw : qw), q2 = a == b ? p2 : v[o];
+        const double x = p1 * q1 + p2 * q2;
+        if (lane < 9) s_Q[lane] = a == b ? 1.0 - 2.0 * x : 2.0 * x;
+    } else if (w == 3) {
+        if (lit && lvlh) {
+            // columns of L: x_b = y_b x z_b, y_b = -h / |h|, h = r x v, z_b = -r / |r|
+            const double hc = y[k1] * y[3 + k2] - y[k2] * y[3 + k1];
+            const double h0 = shfl(hc, 0), h1 = shfl(hc, 1), h2 = shfl(hc, 2);
+            const bool hv = lane & 1;
+            const double m0 = hv ? h0 : y[0], m1 = hv ? h1 : y[1], m2 = hv ? h2 : y[2];
+            const double q = -1.0 / sqrt(m0 * m0 + m1 * m1 + m2 * m2);
+            const double irn = shfl(q, 0), ihn = shfl(q, 1);
+            const double zb = y[c3] * irn, yb = hc * ihn;
+            const double xb = shfl(yb, k1) * shfl(zb, k2) - shfl(yb, k2) * shfl(zb, k1);
+            if (lane < 3) { s_L[3 * lane] = xb; s_L[3 * lane + 1] = yb; s_L[3 * lane + 2] = zb; }
+            if (lane < 2) s_in[lane] = q;
         }
-        double sd = shb[0] * sh[0] + shb[1] * sh[1] + shb[2] * sh[2];
-        for (int k = 0; k < 3; k++) {
-            double wb = (shb[k] - sd * sh[k]) * iwn + g_dist[i] * sh[k] * (1.0 / kAU);
-            rb[k] -= wb;
+        if (P.central == 0 && P.sun3) {
+            const double dc = s_rs[c3] - y[c3];
+            const double d0 = shfl(dc, 0), d1 = shfl(dc, 1), d2c = shfl(dc, 2);
+            const double d2 = d0 * d0 + d1 * d1 + d2c * d2c, dn = sqrt(d2);
+            const double da = d0 * ab[0] + d1 * ab[1] + d2c * ab[2];
+            const double id3 = 1.0 / (d2 * dn), id5 = id3 / d2;
+            const double x = -kMuSun * (ab[c3] * id3 - 3.0 * dc * da * id5);
+            if (lane < 3) s_third[lane] = x;
         }
-        // attitude: R = Q(q) or R = L(y) Q(q)
-        double Q[9], L[9], Qb[9];
-        quat_matrix(P.q, Q);
-        if (P.attitude == 1) {
-            for (int k = 0; k < 9; k++) Qb[k] = Rb[k];
-        } else {
-            lvlh_matrix(y, L);
-            double Lb[9];
-            for (int a = 0; a < 3; a++)
-                for (int b = 0; b < 3; b++) {
-                    double x = 0.0, z = 0.0;
-                    for (int c = 0; c < 3; c++) {
-                        x += L[3 * c + a] * Rb[3 * c + b];  // Qb = L^T Rb
-                        z += Rb[3 * a + c] * Q[3 * b + c];  // Lb = Rb Q^T
-                    }
-                    Qb[3 * a + b] = x;
-                    Lb[3 * a + b] = z;
-                }
-            // L = [x_b y_b z_b]: x_b = y_b x z_b, y_b = -h / |h|, h = r x v, z_b = -r / |r|
-            double yb[3] = {L[1], L[4], L[7]}, zb[3] = {L[2], L[5], L[8]};
-            double xbb[3] = {Lb[0], Lb[3], Lb[6]}, ybb[3] = {Lb[1], Lb[4], Lb[7]}, zbb[3] = {Lb[2], Lb[5], Lb[8]};
-            ybb[0] += zb[1] * xbb[2] - zb[2] * xbb[1];
-            ybb[1] += zb[2] * xbb[0] - zb[0] * xbb[2];
-            ybb[2] += zb[0] * xbb[1] - zb[1] * xbb[0];
-            zbb[0] += xbb[1] * yb[2] - xbb[2] * yb[1];
-            zbb[1] += xbb[2] * yb[0] - xbb[0] * yb[2];
-            zbb[2] += xbb[0] * yb[1] - xbb[1] * yb[0];
-            const double *v = y + 3;
-            double hv[3] = {y[1] * v[2] - y[2] * v[1], y[2] * v[0] - y[0] * v[2], y[0] * v[1] - y[1] * v[0]};
-            double hn = sqrt(hv[0] * hv[0] + hv[1] * hv[1] + hv[2] * hv[2]);
-            const double ihn = 1.0 / hn;
-            double hh[3] = {hv[0] * ihn, hv[1] * ihn, hv[2] * ihn};
-            double yd = ybb[0] * hh[0] + ybb[1] * hh[1] + ybb[2] * hh[2];
-            double hb[3];
-            for (int k = 0; k < 3; k++) hb[k] = -(ybb[k] - yd * hh[k]) * ihn;
-            rb[0] += v[1] * hb[2] - v[2] * hb[1];
-            rb[1] += v[2] * hb[0] - v[0] * hb[2];
-            rb[2] += v[0] * hb[1] - v[1] * hb[0];
-            vb[0] += hb[1] * y[2] - hb[2] * y[1];
-            vb[1] += hb[2] * y[0] - hb[0] * y[2];
-            vb[2] += hb[0] * y[1] - hb[1] * y[0];
-            double rn = sqrt(y[0] * y[0] + y[1] * y[1] + y[2] * y[2]);
-            const double irn = 1.0 / rn;
-            double rh[3] = {y[0] * irn, y[1] * irn, y[2] * irn};
-            double zd = zbb[0] * rh[0] + zbb[1] * rh[1] + zbb[2] * rh[2];
-            for (int k = 0; k < 3; k++) rb[k] += -(zbb[k] - zd * rh[k]) * irn;
-        }
-        // Q of the normalised quaternion, differentiated
-        double g[4];
-        quat_matrix_vjp(P.q, Qb, g);
-        for (int k = 0; k < 4; k++) X.qbar[k] += g[k];
     }
-    for (int k = 0; k < 3; k++) { X.ybar[stage][k] = rb[k]; X.ybar[stage][3 + k] = vb[k]; }
+    __syncthreads();
+    if (lit && lvlh) {
+        // attitude: R = L(y) Q(q): Qb = L^T Rb, Lb = Rb Q^T
+        if (w == 1) {
+            const double z = s_Rb[3 * a] * s_Q[3 * b] + s_Rb[3 * a + 1] * s_Q[3 * b + 1] + s_Rb[3 * a + 2] * s_Q[3 * b + 2];
+            if (lane < 9) s_Lb[lane] = z;
+            __syncwarp();
+            const double irn = -s_in[0], ihn = -s_in[1];
+            const auto col = [&](const double *M, int row, int c) { return M[3 * row + c]; };
+            const double ybb = s_Lb[3 * c3 + 1] + (col(s_L, k1, 2) * col(s_Lb, k2, 0) - col(s_L, k2, 2) * col(s_Lb, k1, 0));
+            const double zbb = s_Lb[3 * c3 + 2] + (col(s_Lb, k1, 0) * col(s_L, k2, 1) - col(s_Lb, k2, 0) * col(s_L, k1, 1));
+            const double hh = -s_L[3 * c3 + 1];  // h / |h|
+            const double yd = shfl(ybb, 0) * shfl(hh, 0) + shfl(ybb, 1) * shfl(hh, 1) + shfl(ybb, 2) * shfl(hh, 2);
+            const double hb = -(ybb - yd * hh) * ihn;
+            const double hb1 = shfl(hb, k1), hb2 = shfl(hb, k2);
+            const double rh = -s_L[3 * c3 + 2];  // r / |r|
+            const double zd = shfl(zbb, 0) * shfl(rh, 0) + shfl(zbb, 1) * shfl(rh, 1) + shfl(zbb, 2) * shfl(rh, 2);
+            const double rb = (y[3 + k1] * hb2 - y[3 + k2] * hb1) - (zbb - zd * rh) * irn;
+            const double vb = hb1 * y[k2] - hb2 * y[k1];
+            if (lane < 3) { s_rv[lane] = rb; s_rv[3 + lane] = vb; }
+        } else if (w == 2) {
+            const double x = s_L[a] * s_Rb[b] + s_L[3 + a] * s_Rb[3 + b] + s_L[6 + a] * s_Rb[6 + b];
+            if (lane < 9) s_Qb[lane] = x;
+        }
+        __syncwarp();
+    }
+    if (w == 2 && lit) {
+        // Q of the normalised quaternion, differentiated
+        const double q0 = shfl(qk, 0), q1 = shfl(qk, 1), q2 = shfl(qk, 2), q3 = shfl(qk, 3);
+        double g[4];
+        quat_unit_vjp(q0, q1, q2, q3, lvlh ? s_Qb : s_Rb, g);
+        const double gd = g[0] * q0 + g[1] * q1 + g[2] * q2 + g[3] * q3;
+        const double gk = lane == 0 ? g[0] : lane == 1 ? g[1] : lane == 2 ? g[2] : g[3];
+        const double x = (gk - gd * qk) / qn;
+        if (lane < 4) X.qbar[lane] += x;
+    }
+    __syncthreads();
+    if (threadIdx.x < 6) {
+        const bool pos = lane < 3;
+        double x = pos ? s_grav[c3] : X.kbar[c3];  // x' = v
+        if (pos && P.central == 0 && P.sun3) x += s_third[c3];
+        if (pos && lit) x -= s_wb[c3];
+        if (lit && lvlh) x += s_rv[lane];
+        X.ybar[stage][lane] = x;
+    }
 }
 
 // attitude quaternion cotangent summed over the trajectories, in order
@@ -793,14 +813,12 @@ cudaError_t launch_prop_record(const PropState *S, int n, const double *sun, con
 cudaError_t launch_adj_prop_in(int n, const PropDev &P, int stage, const StageRec *rec, PropAdj *A, double *g_force,
                                cudaStream_t st)
 {
-    k_adj_prop_in<<<(n + 63) / 64, 64, 0, st>>>(n, P, stage, rec, A, g_force);
-    return cudaGetLastError();
+    return launch_chained(k_adj_prop_in, dim3(n), dim3(32), 0, st, n, P, stage, rec, A, g_force);
 }
 cudaError_t launch_adj_prop_out(int n, const PropDev &P, int stage, const StageRec *rec, PropAdj *A,
                                 const double *g_sun, const double *g_dist, cudaStream_t st)
 {
-    k_adj_prop_out<<<(n + 63) / 64, 64, 0, st>>>(n, P, stage, rec, A, g_sun, g_dist);
-    return cudaGetLastError();
+    return launch_chained(k_adj_prop_out, dim3(n), dim3(128), 0, st, n, P, stage, rec, A, g_sun, g_dist);
 }
 cudaError_t launch_adj_prop_qsum(int n, const PropAdj *A, double *out, cudaStream_t st)
 {

@@ -77,15 +77,10 @@ __device__ __forceinline__ void quat_matrix(const double *q, double *Q)
     Q[6] = 2.0 * (x * z - w * yy);       Q[7] = 2.0 * (yy * z + w * x);       Q[8] = 1.0 - 2.0 * (x * x + yy * yy);
 }
 
-// Cotangent g[4] of the quaternion q as given (before its normalisation) from
-// the cotangent Qb[9] of its rotation matrix: the derivative of each entry of
-// quat_matrix in the normalised components, then the projection of the
-// normalisation (g is orthogonal to q).
-__device__ __forceinline__ void quat_matrix_vjp(const double *q, const double *Qb, double *out)
+// Derivative of each entry of quat_matrix in the components (w0, x, yy, z) of the
+// normalised quaternion, against the cotangent Qb[9] of the matrix.
+__device__ __forceinline__ void quat_unit_vjp(double w0, double x, double yy, double z, const double *Qb, double *g)
 {
-    double qn = sqrt(q[0] * q[0] + q[1] * q[1] + q[2] * q[2] + q[3] * q[3]);
-    double w0 = q[0] / qn, x = q[1] / qn, yy = q[2] / qn, z = q[3] / qn;
-    double g[4];
     g[0] = -2 * z * Qb[1] + 2 * yy * Qb[2] + 2 * z * Qb[3] - 2 * x * Qb[5] - 2 * yy * Qb[6] + 2 * x * Qb[7];
     g[1] = 2 * yy * Qb[1] + 2 * z * Qb[2] + 2 * yy * Qb[3] - 4 * x * Qb[4] - 2 * w0 * Qb[5] + 2 * z * Qb[6] +
            2 * w0 * Qb[7] - 4 * x * Qb[8];
@@ -93,6 +88,17 @@ __device__ __forceinline__ void quat_matrix_vjp(const double *q, const double *Q
            2 * z * Qb[7] - 4 * yy * Qb[8];
     g[3] = -4 * z * Qb[0] - 2 * w0 * Qb[1] + 2 * x * Qb[2] + 2 * w0 * Qb[3] - 4 * z * Qb[4] + 2 * yy * Qb[5] +
            2 * x * Qb[6] + 2 * yy * Qb[7];
+}
+
+// Cotangent g[4] of the quaternion q as given (before its normalisation) from
+// the cotangent Qb[9] of its rotation matrix: the derivative in the normalised
+// components, then the projection of the normalisation (g is orthogonal to q).
+__device__ __forceinline__ void quat_matrix_vjp(const double *q, const double *Qb, double *out)
+{
+    double qn = sqrt(q[0] * q[0] + q[1] * q[1] + q[2] * q[2] + q[3] * q[3]);
+    double w0 = q[0] / qn, x = q[1] / qn, yy = q[2] / qn, z = q[3] / qn;
+    double g[4];
+    quat_unit_vjp(w0, x, yy, z, Qb, g);
     double qh[4] = {w0, x, yy, z};
     double gd = g[0] * qh[0] + g[1] * qh[1] + g[2] * qh[2] + g[3] * qh[3];
     for (int k = 0; k < 4; k++) out[k] = (g[k] - gd * qh[k]) / qn;
