@@ -91,7 +91,8 @@ struct srp_ctx {
     size_t io_cap = 0;
     int32_t *hits = nullptr;
     size_t hits_cap = 0;
-    int *err_flags = nullptr;
+    int *err_flags = nullptr;                // behind the 16 words of stats
+    unsigned long long *h_stats = nullptr;   // pinned: stats and flags read back
     unsigned long long *stats = nullptr;
     srp_eval_stats last{};
     std::vector<cudaEvent_t> events;  // pool for SRP_EVAL_TIMING
@@ -805,6 +806,18 @@ srp_status eval_enqueue(srp_ctx *ctx, Mesh *m, const srp_eval_params *prm, const
 // Adjoint of evaluations whose hits were recorded earlier: posing and window
 // vertices again (no trace), then the frozen-hit reverse sweep, on `st` with
 // the first lane's slots.  hits: [n][N*N][nseg] original triangle ids.
+// The counters and the error flags of a call, one block on the device: cleared by
+// one memset, read back by one copy into pinned memory, which waits for the stream.
+// (Two memsets and two copies into pageable memory, each staged and waited for by the
+// driver: 15 us more a call.)
+constexpr size_t kResultBytes = 17 * sizeof(unsigned long long);
+cudaError_t clear_results(srp_ctx *ctx, cudaStream_t st) { return cudaMemsetAsync(ctx->stats, 0, kResultBytes, st); }
+cudaError_t fetch_results(srp_ctx *ctx, cudaStream_t st)
+{
+    const cudaError_t e = cudaMemcpyAsync(ctx->h_stats, ctx->stats, kResultBytes, cudaMemcpyDeviceToHost, st);
+    return e == cudaSuccess ? cudaStreamSynchronize(st) : e;
+}
+
 srp_status adj_enqueue(srp_ctx *ctx, Mesh *m, const srp_eval_params *prm, const EvalPlan &pl, int n,
                        const double *d_sun, const double *d_dist, const int32_t *hits, const AdjBatch &ab,
                        cudaStream_t st, int64_t &launches)
@@ -963,12 +976,13 @@ srp_status srp_create(srp_ctx **out, int32_t device, void *cuda_stream)
         }
         ctx->own_stream = true;
     }
-    if (dalloc(&ctx->err_flags, sizeof(int)) != cudaSuccess ||
-        dalloc(&ctx->stats, 16 * sizeof(unsigned long long)) != cudaSuccess ||
+    if (cudaHostAlloc(reinterpret_cast<void **>(&ctx->h_stats), kResultBytes, cudaHostAllocDefault) != cudaSuccess ||
+        dalloc(&ctx->stats, kResultBytes) != cudaSuccess ||
         dalloc(&ctx->prop_done, sizeof(int)) != cudaSuccess) {
         srp_destroy(ctx);
         return SRP_ERR_OOM;
     }
+    ctx->err_flags = reinterpret_cast<int *>(ctx->stats + 16);
     for (int b = 0; b < kLanes; b++)
         if (cudaStreamCreateWithFlags(&ctx->lane[b], cudaStreamNonBlocking) != cudaSuccess ||
             cudaEventCreateWithFlags(&ctx->ev_join[b], cudaEventDisableTiming) != cudaSuccess ||
@@ -1028,8 +1042,8 @@ void srp_destroy(srp_ctx *ctx)
     dfree(ctx->sdesc);
     dfree(ctx->arc_hits);
     dfree(ctx->arc_buf);
-    dfree(ctx->err_flags);
     dfree(ctx->stats);
+    if (ctx->h_stats) cudaFreeHost(ctx->h_stats);
     for (cudaEvent_t e : ctx->events) cudaEventDestroy(e);
     for (int b = 0; b < kLanes; b++) {
         if (ctx->lane[b]) cudaStreamSynchronize(ctx->lane[b]), cudaStreamDestroy(ctx->lane[b]);
@@ -1480,8 +1494,7 @@ srp_status srp_eval_batch(srp_ctx *ctx, int32_t mesh_id, const srp_eval_params *
         CK(ctx, cudaMemcpyAsync(d_dist, sun_dist_au, sizeof(double) * n, cudaMemcpyHostToDevice, st));
     if (quat && !q_dev) CK(ctx, cudaMemcpyAsync(d_q, quat, sizeof(double) * 4 * n, cudaMemcpyHostToDevice, st));
     tm.span(4, t_in0, tm.mark(st));
-    CK(ctx, cudaMemsetAsync(ctx->err_flags, 0, sizeof(int), st));
-    CK(ctx, cudaMemsetAsync(ctx->stats, 0, 16 * sizeof(unsigned long long), st));
+    CK(ctx, clear_results(ctx, st));
     int64_t launches = 0, trace_launches = 0;
     if (quat) {
         CK(ctx, launch_att_in(n, d_q, d_sun, d_sb, nullptr, nullptr, m->mass, st));
@@ -1498,12 +1511,9 @@ srp_status srp_eval_batch(srp_ctx *ctx, int32_t mesh_id, const srp_eval_params *
     if (!f_dev) CK(ctx, cudaMemcpyAsync(force, d_f, sizeof(double) * 3 * n, cudaMemcpyDeviceToHost, st));
     if (!t_dev) CK(ctx, cudaMemcpyAsync(torque, d_t, sizeof(double) * 3 * n, cudaMemcpyDeviceToHost, st));
     tm.span(4, t_out0, tm.mark(st));
-    int flags = 0;
-    unsigned long long stats[16];
-    CK(ctx, cudaMemcpyAsync(&flags, ctx->err_flags, sizeof(int), cudaMemcpyDeviceToHost, st));
-    CK(ctx, cudaMemcpyAsync(stats, ctx->stats, sizeof stats, cudaMemcpyDeviceToHost, st));
-    CK(ctx, cudaStreamSynchronize(st));
-    fill_stats(ctx->last, stats);
+    CK(ctx, fetch_results(ctx, st));
+    const int flags = (int)ctx->h_stats[16];
+    fill_stats(ctx->last, ctx->h_stats);
     ctx->last.launches = launches;
     ctx->last.trace_launches = trace_launches;
     tm.collect(ctx->last);
@@ -1549,8 +1559,7 @@ srp_status srp_propagate(srp_ctx *ctx, int32_t mesh_id, const srp_prop_params *p
     double *d_y0 = d_t + 3 * (size_t)n, *d_t01 = d_y0 + 6 * (size_t)n;
     CK(ctx, cudaMemcpyAsync(d_y0, y0, sizeof(double) * 6 * n, cudaMemcpyDefault, st));
     CK(ctx, cudaMemcpyAsync(d_t01, t0_t1, sizeof(double) * 2 * n, cudaMemcpyDefault, st));
-    CK(ctx, cudaMemsetAsync(ctx->err_flags, 0, sizeof(int), st));
-    CK(ctx, cudaMemsetAsync(ctx->stats, 0, 16 * sizeof(unsigned long long), st));
+    CK(ctx, clear_results(ctx, st));
     CK(ctx, cudaMemsetAsync(ctx->prop_done, 0, sizeof(int), st));
     PropState *S = ctx->prop_state;
     PropDev P = prop_dev(p, m);
@@ -1903,8 +1912,7 @@ srp_status srp_grad(srp_ctx *ctx, int32_t mesh_id, const srp_eval_params *prm, i
         CK(ctx, cudaMemcpyAsync(G + ins[k].off, ins[k].src, sizeof(double) * ins[k].count, cudaMemcpyHostToDevice, st));
         dev[k] = G + ins[k].off;
     }
-    CK(ctx, cudaMemsetAsync(ctx->err_flags, 0, sizeof(int), st));
-    CK(ctx, cudaMemsetAsync(ctx->stats, 0, 16 * sizeof(unsigned long long), st));
+    CK(ctx, clear_results(ctx, st));
     int64_t launches = 0, trace_launches = 0;
     // with a quaternion the evaluation runs on the body-frame direction and the
     // body-frame force cotangent; the attitude is differentiated around it
@@ -1934,12 +1942,9 @@ srp_status srp_grad(srp_ctx *ctx, int32_t mesh_id, const srp_eval_params *prm, i
                  {g_mat, off_sum, (size_t)NM2}, {g_angle, off_sum + NM2, (size_t)NP}, {g_quat, off_gq, 4 * (size_t)n}};
     for (auto &o : outs)
         if (o.dst) CK(ctx, cudaMemcpyAsync(o.dst, G + o.off, sizeof(double) * o.count, cudaMemcpyDefault, st));
-    int flags = 0;
-    unsigned long long stats[16];
-    CK(ctx, cudaMemcpyAsync(&flags, ctx->err_flags, sizeof(int), cudaMemcpyDeviceToHost, st));
-    CK(ctx, cudaMemcpyAsync(stats, ctx->stats, sizeof stats, cudaMemcpyDeviceToHost, st));
-    CK(ctx, cudaStreamSynchronize(st));
-    fill_stats(ctx->last, stats);
+    CK(ctx, fetch_results(ctx, st));
+    const int flags = (int)ctx->h_stats[16];
+    fill_stats(ctx->last, ctx->h_stats);
     ctx->last.launches = launches;
     ctx->last.trace_launches = trace_launches;
     if (flags & kFlagTimeout) return fail(ctx, SRP_ERR_TIMEOUT, "a work-queue wait gave up");
@@ -2013,8 +2018,7 @@ srp_status srp_prop_grad(srp_ctx *ctx, int32_t mesh_id, const srp_prop_params *p
     CK(ctx, cudaMemsetAsync(gT, 0, sizeof(double) * n3, st));
     CK(ctx, cudaMemsetAsync(acc, 0, sizeof(double) * (GE + 4), st));
     CK(ctx, cudaMemsetAsync(A, 0, sizeof(PropAdj) * n, st));
-    CK(ctx, cudaMemsetAsync(ctx->err_flags, 0, sizeof(int), st));
-    CK(ctx, cudaMemsetAsync(ctx->stats, 0, 16 * sizeof(unsigned long long), st));
+    CK(ctx, clear_results(ctx, st));
     CK(ctx, cudaMemsetAsync(ctx->prop_done, 0, sizeof(int), st));
     const PropDev P = prop_dev(p, m);
     CK(ctx, launch_prop_init(S, n, d_y0, d_t01, P, nullptr, ctx->prop_done, st));
@@ -2355,8 +2359,7 @@ srp_status srp_propagate_batch(srp_ctx *ctx, const srp_prop_params *p, int32_t n
     CK(ctx, cudaMemcpyAsync(cfg, hcfg.data(), sizeof(double) * hcfg.size(), cudaMemcpyHostToDevice, st));
     CK(ctx, cudaMemcpyAsync(d_y0, hy.data(), sizeof(double) * hy.size(), cudaMemcpyHostToDevice, st));
     CK(ctx, cudaMemcpyAsync(d_t01, ht.data(), sizeof(double) * ht.size(), cudaMemcpyHostToDevice, st));
-    CK(ctx, cudaMemsetAsync(ctx->err_flags, 0, sizeof(int), st));
-    CK(ctx, cudaMemsetAsync(ctx->stats, 0, 16 * sizeof(unsigned long long), st));
+    CK(ctx, clear_results(ctx, st));
     CK(ctx, cudaMemsetAsync(ctx->prop_done, 0, sizeof(int), st));
     PropDev P{};
     P.method = p->method; P.j2 = p->j2; P.sun3 = p->sun3; P.srp = p->srp;
