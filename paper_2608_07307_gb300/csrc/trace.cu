@@ -1323,6 +1323,8 @@ __device__ __forceinline__ int slot_of_block(const SlotDesc *sd, int S, int g)
     return lo;
 }
 
+__device__ __noinline__ Best32 resolve64_warp(const TraceCtx &B, bool want, int N, int i, int j, int seg, const int *hpt,
+                                              int hps, int skip, Cands cd, Best32 best);
 __device__ __noinline__ Best32 resolve64(const TraceCtx &B, int N, int i, int j, int seg, const int *hpt, int hps,
                                          int skip, Cands cd, Best32 best);
 
@@ -2062,9 +2064,11 @@ __global__ void __launch_bounds__(32 * kFewWarps, kFewBlocksPerSM) k_trace_few(T
                 clean = o.ok != 0;
                 if (o.cn.flags) atomicOr(&F.flags, o.cn.flags);
             }
-            if (clean && cd.n > 0) h = resolve64(B, N, i, j, 0, &F.hpt[0][lane], kTileRays, -1, cd, h);  // rare: settle in FP64
-            live = clean && h.part >= 0;
         }
+        const bool want = live && clean && cd.n > 0;
+        if (__any_sync(0xffffffffu, want))  // settle in FP64
+            h = resolve64_warp(B, want, N, i, j, 0, &F.hpt[0][lane], kTileRays, -1, cd, h);
+        live = live && clean && h.part >= 0;
     }
     float delta = B.delta_p, tau = 0.0f;
     for (int seg = 0;; seg++) {
@@ -2131,10 +2135,11 @@ __global__ void __launch_bounds__(32 * kFewWarps, kFewBlocksPerSM) k_trace_few(T
             Best32 b;
             Counts cn = {0u, 0u, 0u, {0u, 0u, 0u, 0u}, 0};
             const bool ok = walk_warp<false>(B, S, D.mesh, mine, r, skip, gpart, gskip, delta, tau, b, cn, cd);
+            const bool want = mine && ok && cd.n > 0;
+            if (__any_sync(0xffffffffu, want))  // settle in FP64
+                b = resolve64_warp(B, want, N, i0 + (tl & (tw - 1)), j0 + (tl >> lw), seg + 1, &F.hpt[0][tl], kTileRays,
+                                   skip, cd, b);
             if (mine) {
-                if (ok && cd.n > 0)  // rare: settle in FP64
-                    b = resolve64(B, N, i0 + (tl & (tw - 1)), j0 + (tl >> lw), seg + 1, &F.hpt[0][tl], kTileRays,
-                                  skip, cd, b);
                 F.res[tl] = !ok ? -2 : (b.part < 0 ? -1 : (b.part << 24) | b.tl);
                 F.b1[tl] = b.b1;
                 F.b2[tl] = b.b2;
@@ -2380,6 +2385,45 @@ __device__ __forceinline__ void wt64(const Ray64 &r, const double *v, double &U,
     T = U * (r.Sz * Akz) + V * (r.Sz * Bkz) + W * (r.Sz * Ckz);
 }
 
+// The exact (FP64) ray of segment seg > 0: from the pixel centre through the planes of the earlier segments' hits.
+__device__ __forceinline__ void segment_ray64(const TraceCtx &B, double uc, double vc, double w0, int seg, const int *hpt,
+                                              int hps, Ray64 &r)
+{
+    for (int k = 0; k < 3; k++) { r.o[k] = uc * B.u[k] + vc * B.v[k] + w0 * B.d[k]; r.d[k] = B.d[k]; }
+    double v[9];
+    for (int s = 0; s < seg; s++) {
+        // hit point on the plane of the segment's triangle, then the specular direction
+        const int hs = hpt[s * hps];
+        tri_v64(B, hs >> 24, hs & 0xffffff, v);
+        double e1[3], e2[3], m[3], ao[3];
+        for (int k = 0; k < 3; k++) { e1[k] = v[3 + k] - v[k]; e2[k] = v[6 + k] - v[k]; ao[k] = v[k] - r.o[k]; }
+        m[0] = e1[1] * e2[2] - e1[2] * e2[1];
+        m[1] = e1[2] * e2[0] - e1[0] * e2[2];
+        m[2] = e1[0] * e2[1] - e1[1] * e2[0];
+        double dm = r.d[0] * m[0] + r.d[1] * m[1] + r.d[2] * m[2];
+        double t = (ao[0] * m[0] + ao[1] * m[1] + ao[2] * m[2]) / dm;
+        double f = 2.0 * dm / (m[0] * m[0] + m[1] * m[1] + m[2] * m[2]);
+        for (int k = 0; k < 3; k++) { r.o[k] = r.o[k] + t * r.d[k]; r.d[k] = r.d[k] - f * m[k]; }
+    }
+    ray64_setup(r);
+
+}
+
+// The FP64 test of a primary segment, in the view frame: edge functions and scaled depth of triangle tl.
+__device__ __forceinline__ void prim64(const TraceCtx &B, const PartView &pv, int tl, double uc, double vc, double w0,
+                                       double &U, double &V, double &W, double &det, double &T)
+{
+    int4 vi = __ldg(pv.v4 + tl);
+    const double *a = B.vview64 + 3 * (size_t)vi.x, *b = B.vview64 + 3 * (size_t)vi.y,
+                 *q = B.vview64 + 3 * (size_t)vi.z;
+    double Ax = a[0] - uc, Ay = a[1] - vc, Bx = b[0] - uc, By = b[1] - vc, Cx = q[0] - uc, Cy = q[1] - vc;
+    U = __dsub_rn(__dmul_rn(Cx, By), __dmul_rn(Cy, Bx));
+    V = __dsub_rn(__dmul_rn(Ax, Cy), __dmul_rn(Ay, Cx));
+    W = __dsub_rn(__dmul_rn(Bx, Ay), __dmul_rn(By, Ax));
+    det = U + V + W;
+    T = U * (a[2] - w0) + V * (b[2] - w0) + W * (q[2] - w0);
+}
+
 // Settle one segment's uncertain FP32 decisions in FP64: the FP64 test of each
 // candidate and of the nearest certain FP32 hit against the segment's exact
 // ray; the nearest t above the self-hit threshold wins, equal t goes to the
@@ -2403,23 +2447,7 @@ __device__ __noinline__ Best32 resolve64(const TraceCtx &B, int N, int i, int j,
     Ray64 r;
     double tlo = 0.0;
     if (seg > 0) {
-        for (int k = 0; k < 3; k++) { r.o[k] = uc * B.u[k] + vc * B.v[k] + w0 * B.d[k]; r.d[k] = B.d[k]; }
-        double v[9];
-        for (int s = 0; s < seg; s++) {
-            // hit point on the plane of the segment's triangle, then the specular direction
-            const int hs = hpt[s * hps];
-            tri_v64(B, hs >> 24, hs & 0xffffff, v);
-            double e1[3], e2[3], m[3], ao[3];
-            for (int k = 0; k < 3; k++) { e1[k] = v[3 + k] - v[k]; e2[k] = v[6 + k] - v[k]; ao[k] = v[k] - r.o[k]; }
-            m[0] = e1[1] * e2[2] - e1[2] * e2[1];
-            m[1] = e1[2] * e2[0] - e1[0] * e2[2];
-            m[2] = e1[0] * e2[1] - e1[1] * e2[0];
-            double dm = r.d[0] * m[0] + r.d[1] * m[1] + r.d[2] * m[2];
-            double t = (ao[0] * m[0] + ao[1] * m[1] + ao[2] * m[2]) / dm;
-            double f = 2.0 * dm / (m[0] * m[0] + m[1] * m[1] + m[2] * m[2]);
-            for (int k = 0; k < 3; k++) { r.o[k] = r.o[k] + t * r.d[k]; r.d[k] = r.d[k] - f * m[k]; }
-        }
-        ray64_setup(r);
+        segment_ray64(B, uc, vc, w0, seg, hpt, hps, r);
         tlo = B.eps;
     }
     for (int c = 0; c <= cd.n; c++) {
@@ -2432,15 +2460,7 @@ __device__ __noinline__ Best32 resolve64(const TraceCtx &B, int N, int i, int j,
         if (orig == skip) continue;
         double U, V, W, det, T;
         if (seg == 0) {
-            int4 vi = __ldg(pv.v4 + tl);
-            const double *a = B.vview64 + 3 * (size_t)vi.x, *b = B.vview64 + 3 * (size_t)vi.y,
-                         *q = B.vview64 + 3 * (size_t)vi.z;
-            double Ax = a[0] - uc, Ay = a[1] - vc, Bx = b[0] - uc, By = b[1] - vc, Cx = q[0] - uc, Cy = q[1] - vc;
-            U = __dsub_rn(__dmul_rn(Cx, By), __dmul_rn(Cy, Bx));
-            V = __dsub_rn(__dmul_rn(Ax, Cy), __dmul_rn(Ay, Cx));
-            W = __dsub_rn(__dmul_rn(Bx, Ay), __dmul_rn(By, Ax));
-            det = U + V + W;
-            T = U * (a[2] - w0) + V * (b[2] - w0) + W * (q[2] - w0);
+            prim64(B, pv, tl, uc, vc, w0, U, V, W, det, T);
         } else {
             double v[9];
             tri_v64(B, p, tl, v);
@@ -2457,6 +2477,85 @@ __device__ __noinline__ Best32 resolve64(const TraceCtx &B, int N, int i, int j,
     best.tl = btl;
     best.b1 = bp >= 0 ? (float)(bV / bU) : 0.f;
     best.b2 = bp >= 0 ? (float)(bW / bU) : 0.f;
+    return best;
+}
+
+// resolve64 by a warp (every lane calls it; `want` where the lane's ray has candidates): the
+// (ray, triangle) pairs are dealt to the lanes, so a step of FP64 tests covers up to 32 of
+// them.  An FP64 instruction takes the warp 64 cycles for one lane or for all: a ray with
+// three triangles to test costs 150 of them instead of 270.  The same decisions, by the same tests.
+__device__ __noinline__ Best32 resolve64_warp(const TraceCtx &B, bool want, int N, int i, int j, int seg, const int *hpt,
+                                              int hps, int skip, Cands cd, Best32 best)
+{
+    constexpr unsigned kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const double uc = B.umin + pix64(((double)i + 0.5) * B.Du, B.rN, N);
+    const double vc = B.vmin + pix64(((double)j + 0.5) * B.Dv, B.rN, N);
+    const double w0 = B.wmin - kStandoff, tlo = seg > 0 ? B.eps : 0.0;
+    Ray64 r;
+    r.o[0] = uc; r.o[1] = vc; r.o[2] = 0.0;
+    r.Sx = r.Sy = r.Sz = 0.0;
+    r.kx = r.ky = r.kz = 0;
+    if (seg > 0 && want) segment_ray64(B, uc, vc, w0, seg, hpt, hps, r);
+    // the lane's pairs: its candidates, then its nearest certain hit
+    const int mine = want ? cd.n + (best.part >= 0 ? 1 : 0) : 0;
+    int end = mine;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(kAll, end, o);
+        if (lane >= o) end += x;
+    }
+    const int first = end - mine, total = __shfl_sync(kAll, end, 31), most = __reduce_max_sync(kAll, mine);
+    const int kk = r.kx | r.ky << 2 | r.kz << 4;
+    const int hit = best.part >= 0 ? (best.part << 24) | best.tl : 0;
+    double bt = INFINITY, bU = 1.0, bV = 0.0, bW = 0.0;
+    int bid = -1, bo = 0x7fffffff;
+    for (int p0 = 0; p0 < total; p0 += 32) {
+        const int p = min(p0 + lane, total - 1);
+        int src = 0;  // the lane whose pair it is: the first with end > p
+        for (int h = 16; h; h >>= 1)
+            if (__shfl_sync(kAll, end, src + h - 1) <= p) src += h;
+        const int c = p - __shfl_sync(kAll, first, src), cn = __shfl_sync(kAll, cd.n, src);
+        const unsigned long long col = __shfl_sync(kAll, reinterpret_cast<unsigned long long>(cd.id), src);
+        const int sh = __shfl_sync(kAll, hit, src), sk = __shfl_sync(kAll, skip, src), k = __shfl_sync(kAll, kk, src);
+        Ray64 q;
+        for (int x = 0; x < 3; x++) q.o[x] = __shfl_sync(kAll, r.o[x], src);
+        q.Sx = __shfl_sync(kAll, r.Sx, src); q.Sy = __shfl_sync(kAll, r.Sy, src); q.Sz = __shfl_sync(kAll, r.Sz, src);
+        q.kx = k & 3; q.ky = (k >> 2) & 3; q.kz = k >> 4;
+        const int id = c < cn ? reinterpret_cast<const int *>(col)[c * kCandStride] : sh;
+        const PartView &pv = B.part[id >> 24];
+        const int tl = id & 0xffffff;
+        int orig = __float_as_int(__ldg(pv.tri + (size_t)tl * 3).w);
+        double U, V, W, det, T, t = INFINITY;
+        if (seg == 0) {
+            prim64(B, pv, tl, q.o[0], q.o[1], w0, U, V, W, det, T);
+        } else {
+            double v[9];
+            tri_v64(B, id >> 24, tl, v);
+            wt64(q, v, U, V, W, det, T);
+        }
+        if (orig == sk || missed64(U, V, W) || zero64(det)) orig = -1;
+        else t = T / det;
+        // each ray's nearest, in its lane
+        int win = -1;
+        for (int e = 0; e < most; e++) {
+            const int l = first + e - p0;
+            const bool own = e < mine && l >= 0 && l < 32;
+            const double te = __shfl_sync(kAll, t, l & 31);
+            const int oe = __shfl_sync(kAll, orig, l & 31);
+            if (own && oe >= 0 && nearer64(te, oe, tlo, bt, bo)) { bt = te; bo = oe; win = l; }
+        }
+        const double wU = __shfl_sync(kAll, det, win & 31), wV = __shfl_sync(kAll, V, win & 31),
+                     wW = __shfl_sync(kAll, W, win & 31);
+        const int wi = __shfl_sync(kAll, id, win & 31);
+        if (win >= 0) { bU = wU; bV = wV; bW = wW; bid = wi; }
+    }
+    if (want) {
+        best.t = (float)bt;
+        best.part = bid < 0 ? -1 : bid >> 24;
+        best.tl = bid < 0 ? -1 : bid & 0xffffff;
+        best.b1 = bid >= 0 ? (float)(bV / bU) : 0.f;
+        best.b2 = bid >= 0 ? (float)(bW / bU) : 0.f;
+    }
     return best;
 }
 
