@@ -43,12 +43,12 @@ NODE_BYTES, TRI_BYTES = 128, 48  # one 4-wide BVH node, one FP32 triangle record
 # DRAM bytes (read + write) of one k_trace launch of the headline workload (8
 # evaluations), from one ncu capture of the current kernel; None when the kernel
 # changed after the capture
-TRACE_DRAM_BYTES_PER_LAUNCH = 124.2e6 + 20.6e6  # mean of three launches, ncu dram__bytes_read/write.sum
+TRACE_DRAM_BYTES_PER_LAUNCH = 122.5e6 + 21.9e6  # mean of three launches, ncu dram__bytes_read/write.sum
 # the same capture's unit throughputs, % of the GB300's peak for each unit
-TRACE_NCU_PCT_OF_PEAK = {"l1tex": 61.4, "l2": 23.0, "dram": 2.6, "sm_issue_active": 66.3,
-                         "l2_bytes_per_launch": 3.272e9, "l1_bytes_per_launch": 4.678e9}
+TRACE_NCU_PCT_OF_PEAK = {"l1tex": 61.3, "l2": 22.0, "dram": 2.6, "sm_issue_active": 66.1,
+                         "l2_bytes_per_launch": 3.116e9, "l1_bytes_per_launch": 4.751e9}
 # L2 bandwidth implied by that capture: L2 bytes / (L2 throughput % / 100) / duration
-L2_PEAK_GBS = 3.272e9 / 0.2300 / 712.5e-6 / 1e9
+L2_PEAK_GBS = 3.116e9 / 0.2205 / 707.4e-6 / 1e9
 HBM_FALLBACK_GBS = 6800.0  # the profiling recipe's fallback when no measured peak is present
 
 

@@ -239,7 +239,7 @@ struct TraceArgs {
     int raster;
     int rast_tris;               // largest triangle count of a slot's mesh (raster grid width)
     unsigned long long *pix_key; // [S][ray_stride] nearest certain FP32 hit: t bits << 32 | 7 - (uncertain
-                                 // triangles, at most kPixCand + 1) << 29 | part << 24 | tl; ~0 none
+                                 // triangles, at most kPixMax + 1) << 29 | part << 24 | tl; ~0 none
     unsigned *pix_cand;          // [S][ray_stride][kPixCand] the first kPixCand uncertain triangles
     unsigned *pix_over;          // [S][kOverWords] further uncertain triangles of the slot's pixels (slot_over)
     int4 *big;                   // [big_cap] (slot, sorted triangle, chunk column, chunk row): chunks of large

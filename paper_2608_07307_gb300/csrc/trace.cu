@@ -771,7 +771,7 @@ __device__ __forceinline__ float min3(float a, float b, float c)
 // place in it from the sorted entry distances of the nodes above its leaf.
 //
 // What bounds it: a batch's chain of dependent fetches, tests and list updates,
-// ~1500 cycles, against ~2700 for a step of 32 one-lane walks, which advances
+// 1900-2650 cycles, against ~2700 for a step of 32 one-lane walks, which advances
 // only the lanes whose rays are still walking.  It issues more instructions in
 // all (nothing is culled, 10-20% more nodes; the lists), so a launch whose tiles
 // fill the GPU many times over is faster with one-lane walks (headline batch 3.95
