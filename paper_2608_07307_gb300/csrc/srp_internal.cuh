@@ -292,7 +292,12 @@ inline bool few_trace(int S, size_t rays, int nseg, bool raster, int n_tris)
     const double r = (double)S * (double)rays;
     return few_slots(S) && nseg > 1 && raster && r * r <= 1.6e7 * (double)n_tris;
 }
-constexpr int kDiffBlocks = 64;  // k_diffuse blocks per slot (fixed: the sums have a fixed order)
+// k_diffuse blocks per slot (fixed: the sums have a fixed order), added in kDiffSums groups (block b in
+// group b mod kDiffSums).  Items cost very different times, and with as many blocks as run at once a
+// launch waits for its slowest; more of them even out as they follow each other.  Eight evaluations of
+// 50k triangles, 256^2, 16 samples a hit, us: 64 blocks 3460, 76 2566, 128 2536, 192 2392, 256 2290,
+// 512 2251, 1024 2280.
+constexpr int kDiffBlocks = 512, kDiffSums = 64;
 // One hit that emits diffuse secondary rays: the FP64 point and lit-side
 // normal from the replay of its ray's specular chain, the weight of one sample
 // (w rho_d / K), the emitting triangle and the sample counter of sample 0.

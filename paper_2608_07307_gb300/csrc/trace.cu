@@ -2956,6 +2956,7 @@ __global__ void __launch_bounds__(kLaneStride) k_demit(TraceArgs a)
     pdl_enter();
     __shared__ TraceCtx B;
     const int s = blockIdx.y;
+    if ((size_t)blockIdx.x * blockDim.x >= (size_t)a.sd[s].N * a.sd[s].N) return;  // no rays (uniform)
     load_ctx(B, a, s);
     __syncthreads();
     const SlotDesc &D = a.sd[s];
@@ -3045,7 +3046,7 @@ __global__ void __launch_bounds__(1024) k_dscan(TraceArgs a)
 // Diffuse rays, step 3: a thread per (record, sample) work item, items in the
 // order of the records (ray-major), each record's K samples consecutive; the
 // record of item e K + q is found by binary search over the prefix.
-// (four blocks an SM, 128 registers: 3.08 ms against 3.57 at three and 3.50 at five)
+// (four blocks an SM, 128 registers: 3.08 ms against 3.57 at three and 3.50 at five, at 64 blocks a slot)
 __global__ void __launch_bounds__(kLaneStride, 4) k_diffuse(TraceArgs a)
 {
     pdl_enter();
@@ -3053,6 +3054,10 @@ __global__ void __launch_bounds__(kLaneStride, 4) k_diffuse(TraceArgs a)
     __shared__ double red[4][6];
     __shared__ __align__(16) WalkShared s_walk[kLaneStride / 32];
     const int s = blockIdx.y;
+    if ((size_t)blockIdx.x * blockDim.x >= (size_t)a.dtot[s] * (size_t)a.n_diffuse) {  // no items (uniform)
+        if (threadIdx.x < 6) a.dpart[((size_t)s * kDiffBlocks + blockIdx.x) * 6 + threadIdx.x] = 0.0;
+        return;
+    }
     load_ctx(B, a, s);
     __syncthreads();
     double acc[6] = {0, 0, 0, 0, 0, 0};
@@ -3304,11 +3309,18 @@ __device__ void final_reduce(const TraceArgs &a, int s, int eval0, double *force
 {
     __shared__ double red2[6][kRed1 / 32];
     __shared__ double s_scale;
+    __shared__ double diff[6][kDiffSums];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = (int)(blockDim.x >> 5);
     const auto first = [&](int b, int k) {
         const double *src = a.partials1 + ((size_t)s * kRed1 + b) * kPart + k;
         return cg ? __ldcg(src) : *src;
     };
+    if (a.n_diffuse > 0 && threadIdx.x < kDiffSums)
+        for (int k = 0; k < 6; k++) {
+            double x = 0.0;
+            for (int b = threadIdx.x; b < kDiffBlocks; b += kDiffSums) x += a.dpart[((size_t)s * kDiffBlocks + b) * 6 + k];
+            diff[k][threadIdx.x] = x;
+        }
     if (w < kRed1 / 32) {
         double v[6];
         for (int k = 0; k < 6; k++) v[k] = first(threadIdx.x, k);
@@ -3347,7 +3359,7 @@ __device__ void final_reduce(const TraceArgs &a, int s, int eval0, double *force
     if (a.sum_mode == 0) {
         for (int q = 0; q < kRed1 / 32; q++) x += red2[k][q];
         if (a.n_diffuse > 0)
-            for (int b = 0; b < kDiffBlocks; b++) x += a.dpart[((size_t)s * kDiffBlocks + b) * 6 + k];
+            for (int g = 0; g < kDiffSums; g++) x += diff[k][g];
     } else {
         // the FP32 modes: the first-level sums again, in order, in FP32
         Comp32 y{0.0f, 0.0f};
@@ -3357,7 +3369,7 @@ __device__ void final_reduce(const TraceArgs &a, int s, int eval0, double *force
         };
         for (int b = 0; b < kRed1; b++) add((float)first(b, k));
         if (a.n_diffuse > 0)
-            for (int b = 0; b < kDiffBlocks; b++) add((float)a.dpart[((size_t)s * kDiffBlocks + b) * 6 + k]);
+            for (int g = 0; g < kDiffSums; g++) add((float)diff[k][g]);
         x = (double)comp_value(y);
     }
     (k < 3 ? force : torque)[3 * (eval0 + s) + k % 3] = x * s_scale;
