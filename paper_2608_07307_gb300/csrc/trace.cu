@@ -2013,6 +2013,7 @@ __global__ void __launch_bounds__(32 * kFewWarps, kFewBlocksPerSM) k_trace_few(T
             F.n_list = some ? 0 : -1;
             F.flags = 0;
         }
+        __syncwarp();  // (lanes add their flags below)
         if (!some) {
             const unsigned n = (unsigned)__popc(__ballot_sync(0xffffffffu, inside));
             if (lane == 0) a.amb_count[tile] = 0;
@@ -2489,6 +2490,7 @@ __device__ __noinline__ Best32 resolve64_warp(const TraceCtx &B, bool want, int 
 {
     constexpr unsigned kAll = 0xffffffffu;
     const int lane = threadIdx.x & 31;
+    __syncwarp();  // the lanes read each other's candidate columns below; votes and shuffles order no memory
     const double uc = B.umin + pix64(((double)i + 0.5) * B.Du, B.rN, N);
     const double vc = B.vmin + pix64(((double)j + 0.5) * B.Dv, B.rN, N);
     const double w0 = B.wmin - kStandoff, tlo = seg > 0 ? B.eps : 0.0;
