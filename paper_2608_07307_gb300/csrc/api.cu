@@ -351,13 +351,13 @@ void coplanar_groups(const std::vector<int> &tris, const int *tri, const std::ve
 // rest-pose box has the largest surface area until it holds four.  A binary
 // node whose leaves are exactly one of the ranges in `pin` is never split into
 // its parent: it heads a 4-wide node of its own, whose part-local ref goes to
-// pin_ref (kEmptyChild where no binary node covers the range).  lp4 gets
+// pin_ref (kNoGroup where no binary node covers the range).  lp4 gets
 // (node << 2) | slot of every leaf.  Returns the depth of the 4-wide tree.
 int collapse_part(const int4 *br, int tc, int tb, const std::vector<int> &svidx, const std::vector<double> &rest,
                   const std::vector<std::pair<int, int>> &pin, std::vector<int> &pin_ref, std::vector<float4> &tmpl,
                   int *lp4)
 {
-    pin_ref.assign(pin.size(), kEmptyChild);
+    pin_ref.assign(pin.size(), kNoGroup);
     if (tc < 2) return 0;
     const int nbin = tc - 1;
     std::vector<int> rlo(nbin), rhi(nbin), pin_of(nbin, -1);
@@ -418,7 +418,7 @@ int collapse_part(const int4 *br, int tc, int tb, const std::vector<int> &svidx,
         todo.pop_back();
         const int me = (int)(tmpl.size() / kNode4) - base;
         if (pin_of[it.bin] >= 0) pin_ref[pin_of[it.bin]] = me;
-        int ch[4] = {br[it.bin].x, br[it.bin].y, kEmptyChild, kEmptyChild};
+        int ch[4] = {br[it.bin].x, br[it.bin].y, 0, 0};
         int n = 2;
         while (n < 4) {
             int best = -1;
@@ -438,6 +438,9 @@ int collapse_part(const int4 *br, int tc, int tb, const std::vector<int> &svidx,
             const float v = (k % 2 == 0) ? finf : -finf;  // lo.x hi.x lo.y hi.y lo.z hi.z: empty
             nd[k] = make_float4(v, v, v, v);
         }
+        // unused slots refer to the part's first triangle: a slab test of numbers never enters their empty box,
+        // one of NaNs enters every box, and a ray that is not a number then stays within the part's arrays too
+        for (int k = n; k < 4; k++) ch[k] = ~0;
         int4 refs = make_int4(ch[0], ch[1], ch[2], ch[3]), meta = make_int4(it.parent, it.slot, n, 0);
         memcpy(&nd[6], &refs, sizeof refs);
         memcpy(&nd[7], &meta, sizeof meta);
@@ -1343,7 +1346,7 @@ srp_status srp_mesh_load(srp_ctx *ctx, const srp_mesh_desc *D, int32_t *mesh_id)
         std::vector<int4> brefs(std::max(nb, 1));
         MK(cudaMemcpy(brefs.data(), node_refs, sizeof(int4) * std::max(nb, 1), cudaMemcpyDeviceToHost));
         std::vector<int> lp4(NT, -1);
-        std::vector<int2> grp(NT, make_int2(kEmptyChild, 0));
+        std::vector<int2> grp(NT, make_int2(kNoGroup, 0));
         std::vector<float4> tmpl;
         int n4 = 0, depth4 = 0;
         const double pose_err = 1e-14 * h.R;  // bound on the FP64 posing error of a vertex
@@ -1370,7 +1373,7 @@ srp_status srp_mesh_load(srp_ctx *ctx, const srp_mesh_desc *D, int32_t *mesh_id)
             int d4 = collapse_part(brefs.data() + bin_begin[p], pi.tri_count, pi.tri_begin, svidx, rest, pin, pin_ref,
                                    tmpl, lp4.data() + pi.tri_begin);
             for (size_t i = 0; i < pin.size(); i++) {
-                if (pin_ref[i] == kEmptyChild) continue;
+                if (pin_ref[i] == kNoGroup) continue;
                 for (int k = pin[i].first; k <= pin[i].second; k++) {
                     const int t = pi.tri_begin + k;
                     const float dev = (float)((tdev[sorig[t]] + pose_err) * 1.001);

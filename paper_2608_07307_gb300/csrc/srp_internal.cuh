@@ -57,7 +57,7 @@ constexpr int kMaxMats = SRP_MAX_MATS;
 constexpr int kMaxBounces = SRP_MAX_BOUNCES;
 constexpr int kStack = 96;          // traversal stack entries (>= 3 x 4-wide tree depth + 1, checked at load)
 constexpr int kNode4 = 8;           // float4 per 4-wide node
-constexpr int kEmptyChild = (int)0x80000000;  // child ref of an unused slot (its box is empty)
+constexpr int kNoGroup = (int)0x80000000;  // no coplanar group (a node ref that no part has)
 constexpr int kTraceThreads = 256;  // 16 x 16 pixel tile per block
 constexpr int kTile = 16;
 constexpr double kStandoff = 1.0;   // ray origins start 1 m in front of the nearest vertex
@@ -168,7 +168,7 @@ struct MeshDev {
     float4 *tri_static;    // [n_static_tris][3]
     float4 *node_static;   // [n_static_nodes][kNode4]
     int2 *grp;             // [n_tris] sorted -> (part-local 4-wide ref of the subtree holding the triangle's
-                           // coplanar group or kEmptyChild, FP32 bits of the group's deviation from its plane
+                           // coplanar group or kNoGroup, FP32 bits of the group's deviation from its plane
                            // plus the posing error bound, metres)
     float2 *mat32;         // [n_mats] (rho_s, rho_d) FP32
     double *mat64;         // [n_mats][2]

@@ -638,7 +638,7 @@ __device__ __forceinline__ bool nearest32(const TraceCtx &B, const Ray32 &r, flo
         if (te[q] > best.t + tau) break;  // this part and every later one start beyond the best hit
         const int p = po[q];
         const PartView &pv = B.part[p];
-        const int gs = p == gpart ? gskip : kEmptyChild;
+        const int gs = p == gpart ? gskip : kNoGroup;
         int sp = 0, iters = 0;
         int ref = pv.root;
         while (true) {
@@ -705,7 +705,7 @@ __device__ __noinline__ Near32 nearest32_primary(const TraceCtx &B, const Ray32 
                                                  float tau, Counts cn, Cands cd)
 {
     Near32 o;
-    o.ok = nearest32<COUNT, true, COPY>(B, r, uc, vc, 0.0f, -1, -1, kEmptyChild, delta, tau, o.b, cn, cd) ? 1 : 0;
+    o.ok = nearest32<COUNT, true, COPY>(B, r, uc, vc, 0.0f, -1, -1, kNoGroup, delta, tau, o.b, cn, cd) ? 1 : 0;
     o.cn = cn;
     o.cand_n = cd.n;
     return o;
@@ -1165,7 +1165,7 @@ __device__ __forceinline__ bool walk_warp(const TraceCtx &B, WalkShared &S, cons
     unsigned nn = 0u, nt = 0u, nf = 0u;  // entries of the three lists
     bool over = fall;                    // (uniform over the warp)
     // the group's packed part and node, or a value no entry has
-    const unsigned gent = gskip == kEmptyChild ? 0xffffffffu : ((unsigned)gpart << rbits) | (unsigned)gskip;
+    const unsigned gent = gskip == kNoGroup ? 0xffffffffu : ((unsigned)gpart << rbits) | (unsigned)gskip;
     if (live) {
         S.ra[lane] = make_float4(r.o[0], r.o[1], r.o[2], __uint_as_float(gent));
         S.rb[lane] = make_float4(r.inv[0], r.inv[1], r.inv[2], __int_as_float(skip));
@@ -1826,7 +1826,7 @@ __device__ __forceinline__ void trace_block(const TraceArgs &a, int vb, TraceCtx
         const float uc = fmaf((float)i + 0.5f, B.du32, B.umin32);
         const float vc = fmaf((float)j + 0.5f, B.dv32, B.vmin32);
         float wgt = 1.0f;
-        int skip = -1, gpart = -1, gskip = kEmptyChild;
+        int skip = -1, gpart = -1, gskip = kNoGroup;
         float acc[6] = {0, 0, 0, 0, 0, 0};
         unsigned hitbits = 0u;
         bool clean = true;
@@ -1904,7 +1904,7 @@ __device__ __forceinline__ void trace_block(const TraceArgs &a, int vb, TraceCtx
             // only be met within dev / |dn| of the origin, inside the self-hit distance eps
             const int2 g = __ldg(B.grp + B.part[h.part].tri_begin + h.tl);
             gpart = h.part;
-            gskip = fabsf(sh.dn) * B.eps32 > 16.0f * __int_as_float(g.y) ? g.x : kEmptyChild;
+            gskip = fabsf(sh.dn) * B.eps32 > 16.0f * __int_as_float(g.y) ? g.x : kNoGroup;
             // next segment: world-frame test; the origin error grows with the previous bound
             delta = B.delta_s + 2.0f * delta;
             tau = 64.0f * delta + 32.0f * kU * (B.R + B.L);
@@ -2095,7 +2095,7 @@ __global__ void __launch_bounds__(32 * kFewWarps, kFewBlocksPerSM) k_trace_few(T
                     // the reflected ray leaves the hit triangle's plane at |dn|: its coplanar group can
                     // only be met within dev / |dn| of the origin, inside the self-hit distance eps
                     const int2 g = __ldg(B.grp + B.part[h.part].tri_begin + h.tl);
-                    F.gskip[lane] = fabsf(sh.dn) * B.eps32 > 16.0f * __int_as_float(g.y) ? g.x : kEmptyChild;
+                    F.gskip[lane] = fabsf(sh.dn) * B.eps32 > 16.0f * __int_as_float(g.y) ? g.x : kNoGroup;
                     ray_setup(r);
                     F.ra[lane] = make_float4(r.o[0], r.o[1], r.o[2], __int_as_float(sh.orig));
                     F.rb[lane] = make_float4(r.inv[0], r.inv[1], r.inv[2], __int_as_float(h.part));
@@ -2121,7 +2121,7 @@ __global__ void __launch_bounds__(32 * kFewWarps, kFewBlocksPerSM) k_trace_few(T
             const bool mine = at < n;
             const int tl = mine ? F.list[at] : 0;
             Ray32 r;
-            int skip = -1, gpart = -1, gskip = kEmptyChild;
+            int skip = -1, gpart = -1, gskip = kNoGroup;
             if (mine) {
                 const float4 A = F.ra[tl], I = F.rb[tl], C = F.rc[tl];
                 r.o[0] = A.x; r.o[1] = A.y; r.o[2] = A.z;
@@ -2900,7 +2900,7 @@ __device__ __forceinline__ void diffuse_sample(const TraceCtx &B, WalkShared &S,
         Cands cd;
         cd.n = 0;
         cd.id = reinterpret_cast<int *>(S.node) + (threadIdx.x & 31);
-        const bool ok = walk_warp<false>(B, S, mesh, live, q, src, -1, kEmptyChild, delta, tau, b, cn, cd);
+        const bool ok = walk_warp<false>(B, S, mesh, live, q, src, -1, kNoGroup, delta, tau, b, cn, cd);
         if (!live) return;
         if (ok) {
             if (cd.n == 0) {
@@ -3449,8 +3449,8 @@ __global__ void k_bvh_check(const unsigned char *tctx, int *tri_seen, unsigned l
             const int4 refs4 = *reinterpret_cast<const int4 *>(n + 6);
             const int rf[4] = {refs4.x, refs4.y, refs4.z, refs4.w};
             nodes++;
-            for (int c = 0; c < 4; c++) {
-                if (rf[c] == kEmptyChild) continue;
+            const int used = reinterpret_cast<const int4 *>(n + 7)->z;  // (the children come first)
+            for (int c = 0; c < used; c++) {
                 float bx[6];
                 for (int k = 0; k < 6; k++) bx[k] = reinterpret_cast<const float *>(n + k)[c];
                 if (!inside(bx, pbox)) outside_box++;
