@@ -124,10 +124,14 @@ int win_blocks(const AdjArgs &a)
 }
 
 // The window's extreme vertex c (0..3) of slot s: the lowest of its G <= 32 blocks', by a warp.
+// No vertex has the bound when every projection is NaN (a Sun direction or quaternion of length
+// zero, or with a component that is not finite): the NaN's ordered image replaces only one of
+// the two starting bounds.  Vertex 0 then stands for it, its projection being NaN like the others'.
 __device__ __forceinline__ int window_vertex(const AdjArgs &a, int s, int c, int G)
 {
     const int lane = threadIdx.x & 31;
-    return __reduce_min_sync(kFull, lane < G ? a.win_pid[((size_t)s * G + lane) * 4 + c] : INT_MAX);
+    const int id = __reduce_min_sync(kFull, lane < G ? a.win_pid[((size_t)s * G + lane) * 4 + c] : INT_MAX);
+    return id == INT_MAX ? 0 : id;
 }
 
 // --------------------------------------------------------------- rays

@@ -47,3 +47,27 @@ def test_rays_that_are_not_numbers_stay_in_the_tree(ctx, mesh, n, k, opts):
     b = ctx.eval_batch(mid, s, N=48, bounces=1, hits=True, **kw)
     assert all(np.array_equal(x, y) for x, y in zip(a, b))
     ctx.free_mesh(mid)
+
+
+# the window search of the gradient: no vertex has the bound of projections that are all NaN
+@pytest.mark.parametrize("mesh", list(MESHES))
+@pytest.mark.parametrize("bad", ["zero", "negative_nan", "inf"])
+@pytest.mark.parametrize("n, k", [(1, 0), (3, 2), (6, 0)])
+def test_gradient_of_a_degenerate_direction(ctx, mesh, bad, n, k):
+    m = MESHES[mesh]()
+    mid = ctx.load_mesh(m)
+    rng = np.random.default_rng(n)
+    s, gF, gT = I.sun_dirs_uniform(n, seed=5), rng.normal(size=(n, 3)), rng.normal(size=(n, 3))
+    a = ctx.grad(mid, s, gF, gT, N=48, bounces=1)
+    t = s.copy()
+    t[k] = BAD[bad]
+    b = ctx.grad(mid, t, gF, gT, N=48, bounces=1)
+    keep = [e for e in range(n) if e != k]
+    for name in ("F", "T", "sun"):
+        assert np.isnan(b[name][k]).all(), (name, b[name][k])
+        assert np.array_equal(a[name][keep], b[name][keep]), name
+    assert np.isnan(b["mat"]).any()  # sums over the evaluations
+    c = ctx.grad(mid, s, gF, gT, N=48, bounces=1)
+    for name in a:
+        assert np.array_equal(a[name], c[name]), name
+    ctx.free_mesh(mid)
