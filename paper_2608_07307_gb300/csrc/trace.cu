@@ -236,8 +236,8 @@ __global__ void k_frame(TraceArgs a)
         B.walk_bound = a.walk_limit_test ? 1 : (int)min(64ll * n_tris + 4096ll, 0x7fffffffll);
         if (a.red_ticket) a.red_ticket[s] = 0u;
     }
-    if (skip) return;
-    // the parts' traversal views, a lane each
+    // the parts' traversal views, a lane each (in a skipped slot too: its context is copied by blocks that find out
+    // then, and the copy follows box_src)
     if (lane < np) {
         PartView &pv = B.part[lane];
         pv.root = pi.tri_count > 1 ? 0 : ~0;
@@ -257,6 +257,7 @@ __global__ void k_frame(TraceArgs a)
             pv.box_src = box_static;
         }
     }
+    if (skip) return;
     const auto all = [](double x, int l) { return __shfl_sync(0xffffffffu, x, l); };
     const double umin = all(lo, 0), umax = all(hi, 0), vmin = all(lo, 1), vmax = all(hi, 1), wmin = all(lo, 2),
                  wmax = all(hi, 2);
