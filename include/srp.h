@@ -243,7 +243,10 @@ srp_status srp_set_panel_angles(srp_ctx *ctx, int32_t mesh_id, int32_t n, const 
  * traced for `bounces` more levels (weight times rho_s; a secondary ray never
  * hits the triangle it leaves); sum of all pixels times P0 / dist^2 times the
  * pixel area.
- *   sun_dir_body [n][3]   unit vectors towards the Sun, body frame; with quat,
+ *   sun_dir_body [n][3]   vectors towards the Sun (any length), body frame; one
+ *                         of length zero, or not finite, makes its own outputs
+ *                         NaN (its hits -1, its gradients NaN) and no other;
+ *                         with quat,
  *                         the Sun direction in the inertial frame instead
  *   quat         [n][4]   NULL, or the attitude per evaluation: scalar-first
  *                         quaternion body -> inertial (normalised here).  The

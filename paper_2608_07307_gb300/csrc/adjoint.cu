@@ -426,9 +426,11 @@ __global__ void __launch_bounds__(128) k_adj_finish(AdjArgs a, int runs, int GW)
     const int e = a.eval0 + s, W = a.width, nm2 = 2 * a.n_mats, np = a.n_parts;
     double *ge = a.g_eval + (size_t)e * (nm2 + np);
     if (P.skip) {
-        for (int k = threadIdx.x; k < nm2 + np; k += blockDim.x) ge[k] = 0.0;
-        if (threadIdx.x < 3) a.g_sun[3 * (size_t)e + threadIdx.x] = 0.0;
-        if (threadIdx.x == 0 && a.g_dist) a.g_dist[e] = 0.0;
+        const double x = P.skip == kSkipDir ? (double)NAN : 0.0;
+        for (int k = threadIdx.x; k < nm2 + np; k += blockDim.x)
+            ge[k] = k >= nm2 && !m.part[k - nm2].movable ? 0.0 : x;
+        if (threadIdx.x < 3) a.g_sun[3 * (size_t)e + threadIdx.x] = x;
+        if (threadIdx.x == 0 && a.g_dist) a.g_dist[e] = x;
         return;
     }
     extern __shared__ double tot[];  // [W]

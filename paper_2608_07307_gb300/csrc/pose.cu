@@ -47,7 +47,6 @@ __global__ void __launch_bounds__(kPoseThreads) k_pose(const SlotDesc *sd, const
     const int e = eval0 + slot;
     double s[3] = {sun_dirs[3 * e], sun_dirs[3 * e + 1], sun_dirs[3 * e + 2]};
     const double dist = sun_dist ? sun_dist[e] : 1.0;
-    const int skip = dist < 0.0 ? 1 : 0;  // a negative distance asks to skip this evaluation
     const int np = mesh->n_parts;
     // depth of each part in the kinematic tree (parents precede children), a part a lane
     const int par_l = (lane < np && lane > 0) ? mesh->part[lane].parent : -1;
@@ -65,6 +64,10 @@ __global__ void __launch_bounds__(kPoseThreads) k_pose(const SlotDesc *sd, const
         const double x = (c3 == 0 ? s[0] : c3 == 1 ? s[1] : s[2]) / sn;
         for (int k = 0; k < 3; k++) s[k] = group_shfl(x, k);
     }
+    // the largest component of a direction lies in [0.5, 2) (by its high word; above it: infinity, NaN)
+    int top = 0;
+    for (int k = 0; k < 3; k++) top = max(top, __double2hiint(s[k]) & 0x7fffffff);
+    const int skip = dist < 0.0 ? kSkipDist : (top >= 0x3fe00000 && top < 0x40000000) ? 0 : kSkipDir;
     if (threadIdx.x == 0) {
         s_track = s_free = 0u;
         P.eval = e;

@@ -60,6 +60,9 @@ constexpr int kNode4 = 8;           // float4 per 4-wide node
 constexpr int kNoGroup = (int)0x80000000;  // no coplanar group (a node ref that no part has)
 constexpr int kTraceThreads = 256;  // 16 x 16 pixel tile per block
 constexpr int kTile = 16;
+// SlotPose.skip: why a slot is not evaluated.  A distance below zero asks for it (zero outputs); a direction
+// that has none (length zero, not finite) gives NaN, without rays that are not numbers walking the tree.
+constexpr int kSkipDist = 1, kSkipDir = 2;
 constexpr double kStandoff = 1.0;   // ray origins start 1 m in front of the nearest vertex
 
 // Device error flags (bits of SlotPose::flags / the context error word).
@@ -132,7 +135,7 @@ struct SlotPose {
     double scale;             // P0 / dist^2 (multiplied by the pixel area at the end)
     int eval;                 // evaluation index in the batch
     int flags;                // device error flags
-    int skip;                 // evaluation skipped (negative Sun distance): every later kernel returns early
+    int skip;                 // evaluation skipped (kSkip...): every later kernel returns early
     unsigned free_mask;       // bit p: joint p is movable and its angle lies strictly inside its limits
     unsigned track_mask;      // bit p: joint p's angle follows the Sun (tracking, non-degenerate)
     double s_norm;            // length of the Sun direction as given

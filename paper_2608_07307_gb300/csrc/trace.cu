@@ -120,7 +120,7 @@ struct TraceCtx {
     int ref_bits;          // bits of a node or triangle in a walk entry (walk_warp); 0: a part has too many
     int walk_bound;        // bound on the batches of a walk
     int walk_spare;        // node list entries kept for a depth-first walk at the end of the room
-    int skip;              // evaluation skipped: trace blocks only clear their hand-off count
+    int skip;              // evaluation skipped (kSkip...): trace blocks only clear their hand-off count
     const float4 *vview;   // slot's view-frame vertices
     const double *vview64; // the same in FP64
     const float2 *mat32;
@@ -1797,13 +1797,15 @@ __device__ __forceinline__ void trace_block(const TraceArgs &a, int vb, TraceCtx
         const size_t tile = (size_t)s * a.n_blocks_x + tile_id;
         const unsigned n = (unsigned)__popc(__ballot_sync(0xffffffffu, inside));
         if (lane == 0) a.amb_count[tile] = 0;
-        if (reinterpret_cast<const TraceCtx *>(a.tctx)[s].skip) return;
-        if (lane < 6) a.partials[tile * 6 + lane] = 0.0f;
-        if (lane < (COUNT ? kCnt : 7)) a.pcounts[tile * kCnt + lane] = lane == 1 ? n : 0u;  // (segments)
+        const int skip = reinterpret_cast<const TraceCtx *>(a.tctx)[s].skip;
+        if (skip == kSkipDist) return;
         if (HITS && inside) {
             int32_t *hq = a.hits + ((size_t)s * a.ray_stride + (size_t)i * N + j) * a.seg_stride;
             for (int k = 0; k < nseg; k++) hq[k] = -1;
         }
+        if (skip) return;
+        if (lane < 6) a.partials[tile * 6 + lane] = 0.0f;
+        if (lane < (COUNT ? kCnt : 7)) a.pcounts[tile * kCnt + lane] = lane == 1 ? n : 0u;  // (segments)
         return;
     }
     load_ctx(B, a, s);
@@ -1811,6 +1813,10 @@ __device__ __forceinline__ void trace_block(const TraceArgs &a, int vb, TraceCtx
     if (tile_id >= D.tiles) return;
     if (B.skip) {
         if (lane == 0) a.amb_count[(size_t)s * a.n_blocks_x + tile_id] = 0;
+        if (HITS && inside && B.skip == kSkipDir) {
+            int32_t *hq = a.hits + ((size_t)s * a.ray_stride + (size_t)i * N + j) * a.seg_stride;
+            for (int k = 0; k < nseg; k++) hq[k] = -1;
+        }
         return;
     }
     // per-ray results: force / torque in FP32 (at most 1 + bounces terms); counts
@@ -2006,7 +2012,7 @@ __global__ void __launch_bounds__(32 * kFewWarps, kFewBlocksPerSM) k_trace_few(T
         live = seen = inside && !skip_slot && (bad || pk != ~0ull);  // (all ones: no hit, no candidate)
         nseg_done = inside ? 1 : 0;
         const bool some = __any_sync(0xffffffffu, live);
-        if (HITS && inside && !skip_slot && !live) {
+        if (HITS && inside && B.skip != kSkipDist && !live) {
             int32_t *hq = a.hits + (px0 + ray) * a.seg_stride;
             for (int k = 0; k < nseg; k++) hq[k] = -1;
         }
@@ -3186,14 +3192,28 @@ __device__ __noinline__ void refine_block(const TraceCtx &B, const TraceArgs &a,
     }
 }
 
+// The outputs of an evaluation that was not run: zero force and torque, or NaN (and its rays
+// counted, each a segment without a hit) where it had no Sun direction.
+__device__ __forceinline__ void skipped_outputs(const TraceArgs &a, int s, int eval0, double *force, double *torque,
+                                                unsigned long long *stats_accum)
+{
+    const bool dir = a.pose[s].skip == kSkipDir;
+    if (threadIdx.x < 6) (threadIdx.x < 3 ? force : torque)[3 * (eval0 + s) + threadIdx.x % 3] = dir ? (double)NAN : 0.0;
+    if (dir && stats_accum && threadIdx.x == 0) {
+        const unsigned long long N = (unsigned long long)a.sd[s].N;
+        atomicAdd(&stats_accum[0], 1ull);
+        atomicAdd(&stats_accum[1], N * N);
+        atomicAdd(&stats_accum[3], N * N);
+    }
+}
+
 __global__ void __launch_bounds__(32 * kRedWarps, kRedBlocksPerSM) k_reduce1(TraceArgs a, int eval0, double *force, double *torque,
                                                  int *err_flags, unsigned long long *stats_accum, int fuse)
 {
     pdl_enter();
     const int s = blockIdx.y, b = blockIdx.x;
     if (a.pose[s].skip) {  // uniform over the block
-        // a skipped evaluation outputs zero force and torque
-        if (fuse && b == 0 && threadIdx.x < 6) (threadIdx.x < 3 ? force : torque)[3 * (eval0 + s) + threadIdx.x % 3] = 0.0;
+        if (fuse && b == 0) skipped_outputs(a, s, eval0, force, torque, stats_accum);
         return;
     }
     const int nt = a.sd[s].tiles;
@@ -3385,8 +3405,7 @@ __global__ void __launch_bounds__(kRed1) k_reduce(TraceArgs a, int eval0, double
     pdl_enter();
     const int s = blockIdx.x;
     if (a.pose[s].skip) {
-        // a skipped evaluation outputs zero force and torque
-        if (threadIdx.x < 6) (threadIdx.x < 3 ? force : torque)[3 * (eval0 + s) + threadIdx.x % 3] = 0.0;
+        skipped_outputs(a, s, eval0, force, torque, stats_accum);
         return;
     }
     final_reduce(a, s, eval0, force, torque, err_flags, stats_accum, false);
