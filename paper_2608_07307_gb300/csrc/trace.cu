@@ -1717,6 +1717,10 @@ __device__ __forceinline__ Shade32 shade_hit(const TraceCtx &B, const Best32 &h,
     return o;
 }
 
+// A triangle whose edges' cross product, or its square, underflows in FP32 (a sliver of 1e-23 m^2, or
+// vertices that round to one line) has no FP32 normal: the ray goes to the FP64 re-trace, which has one.
+__device__ __forceinline__ bool no_normal(const Shade32 &s) { return !(fabsf(s.dn) < 2.0f); }
+
 // What a tile's 32 rays leave, by one warp, a lane a ray: the list of the rays
 // handed to the FP64 path, force and torque, counts.
 template <bool COUNT>
@@ -1900,6 +1904,7 @@ __device__ __forceinline__ void trace_block(const TraceArgs &a, int vb, TraceCtx
             hpt[seg * kLaneStride] = (h.part << 24) | h.tl;
             hitbits |= 1u << seg;
             const Shade32 sh = shade_hit(B, h, r.d, wgt, acc);
+            if (no_normal(sh)) { clean = false; break; }
             wgt *= sh.rs;
             if (seg + 1 >= nseg || wgt == 0.0f) break;
             for (int k = 0; k < 3; k++) {
@@ -2090,8 +2095,9 @@ __global__ void __launch_bounds__(32 * kFewWarps, kFewBlocksPerSM) k_trace_few(T
                 for (int k = 0; k < 3; k++) d[k] = F.d[k][lane];
                 const Shade32 sh = shade_hit(B, h, d, wgt, acc);
                 for (int k = 0; k < 6; k++) F.acc[k][lane] = acc[k];
+                clean = !no_normal(sh);
                 wgt *= sh.rs;
-                live = seg + 1 < nseg && wgt != 0.0f;
+                live = clean && seg + 1 < nseg && wgt != 0.0f;
                 if (live) {
                     Ray32 r;
                     for (int k = 0; k < 3; k++) {
