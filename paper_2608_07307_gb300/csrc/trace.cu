@@ -1443,11 +1443,20 @@ __device__ __forceinline__ unsigned key_cands(unsigned long long k) { return 7u 
 // word, then (pixel, triangle) pairs; reset by the frame kernel.
 __device__ __forceinline__ unsigned *slot_over(const TraceArgs &a, int s) { return a.pix_over + (size_t)s * kOverWords; }
 
+// Are the pn candidates of a pixel all listed (else its ray traverses)?  Past
+// kPixCand they are while the slot's list holds those of all its pixels: which
+// entries a list that ran over has lost depends on the order of arrival, how many
+// were counted does not, so such a list counts for none of the pixels.
+__device__ __forceinline__ bool pix_listed(unsigned pn, const unsigned *over)
+{
+    return pn <= (unsigned)kPixCand || (pn <= (unsigned)kPixMax && __ldcg(over) <= (unsigned)kOverCap);
+}
+
 // A pixel's candidates past the first kPixCand into the ray's column (out of
 // line: rare); returns how many candidates the column holds.
 __device__ __noinline__ int over_cands(const unsigned *over, unsigned pix, int pn, int *col)
 {
-    const int n = (int)min(__ldcg(over), (unsigned)kOverCap);
+    const int n = (int)__ldcg(over);  // (pix_listed: at most kOverCap)
     int at = kPixCand;
     for (int k = 0; k < n; k++) {
         const uint2 e = __ldcg(reinterpret_cast<const uint2 *>(over) + 1 + k);
@@ -1509,9 +1518,9 @@ __device__ __forceinline__ void rast_pixel(const RastView &V, unsigned long long
             cand[px * kPixCand + slot] = id;
         } else if (slot < kPixMax) {
             // a pixel on a vertex shared by several triangles (rare): the slot's own list of such
+            // (counted past its end too: see pix_listed)
             const unsigned at = atomicAdd(over, 1u);
             if (at < (unsigned)kOverCap) reinterpret_cast<uint2 *>(over)[1 + at] = make_uint2((unsigned)px, id);
-            else atomicAnd(key + px, ~(7ull << kKeyField));
         }
     }
 }
@@ -1850,7 +1859,7 @@ __device__ __forceinline__ void trace_block(const TraceArgs &a, int vb, TraceCtx
         if (a.raster) {
             const size_t px = (size_t)s * a.ray_stride + ray;
             const unsigned pn = key_cands(pk);
-            rast = pn <= (unsigned)kPixMax && !bad;
+            rast = !bad && pix_listed(pn, slot_over(a, s));
             if (rast) {
                 cd.n = (int)pn;
                 for (int c = 0; c < min((int)pn, kPixCand); c++)
@@ -2042,7 +2051,7 @@ __global__ void __launch_bounds__(32 * kFewWarps, kFewBlocksPerSM) k_trace_few(T
             const float uc = fmaf((float)i + 0.5f, B.du32, B.umin32);
             const float vc = fmaf((float)j + 0.5f, B.dv32, B.vmin32);
             const unsigned pn = key_cands(pk);
-            if (pn <= (unsigned)kPixMax && !bad) {
+            if (!bad && pix_listed(pn, slot_over(a, s))) {
                 if (!key_none(pk)) {
                     // the raster's nearest certain hit; its barycentric weights as the traversal forms them
                     const unsigned id = (unsigned)pk & kKeyId;
