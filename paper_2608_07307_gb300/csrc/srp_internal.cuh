@@ -211,6 +211,7 @@ struct SlotDesc {
 //   edge, near tie, self-hit band).
 constexpr int kPart = 20;
 constexpr int kCnt = kPart - 6;  // the integer counts (6..19) of a tile partial
+constexpr int kCntRay = 3 + kMaxBounces;  // of which always written: hand-offs, segments, hits per level
 
 // Arguments of the trace / refine kernels.  A trace warp covers one tile of
 // kTileRays rays (4 x 8, 8 x 4, 16 x 2 or 32 x 1 pixels).

@@ -1753,7 +1753,7 @@ __device__ __forceinline__ void tile_results(const TraceArgs &a, int s, int tile
     // counts 0..6 always (hand-offs, segments, hits per segment level); the
     // traversal counters only in the counting variant
 #pragma unroll
-    for (int k = 0; k < (COUNT ? kCnt : 7); k++) {
+    for (int k = 0; k < (COUNT ? kCnt : kCntRay); k++) {
         unsigned v;
         if (k == 0) v = c_handoff;
         else if (k == 1) v = c_segs;
@@ -1818,7 +1818,7 @@ __device__ __forceinline__ void trace_block(const TraceArgs &a, int vb, TraceCtx
         }
         if (skip) return;
         if (lane < 6) a.partials[tile * 6 + lane] = 0.0f;
-        if (lane < (COUNT ? kCnt : 7)) a.pcounts[tile * kCnt + lane] = lane == 1 ? n : 0u;  // (segments)
+        if (lane < (COUNT ? kCnt : kCntRay)) a.pcounts[tile * kCnt + lane] = lane == 1 ? n : 0u;  // (segments)
         return;
     }
     load_ctx(B, a, s);
@@ -2040,7 +2040,7 @@ __global__ void __launch_bounds__(32 * kFewWarps, kFewBlocksPerSM) k_trace_few(T
             if (lane == 0) a.amb_count[tile] = 0;
             if (!skip_slot) {
                 if (lane < 6) a.partials[tile * 6 + lane] = 0.0f;
-                if (lane < 7) a.pcounts[tile * kCnt + lane] = lane == 1 ? n : 0u;  // (segments)
+                if (lane < kCntRay) a.pcounts[tile * kCnt + lane] = lane == 1 ? n : 0u;  // (segments)
             }
         } else {
             for (int k = 0; k < 6; k++) F.acc[k][lane] = 0.0f;
@@ -3239,10 +3239,9 @@ __global__ void __launch_bounds__(32 * kRedWarps, kRedBlocksPerSM) k_reduce1(Tra
     Comp32 f32[6];  // the FP32 sum modes
     for (int k = 0; k < 6; k++) f32[k] = Comp32{0.0f, 0.0f};
     const int mode = a.sum_mode;
-    // counts of one block (at most 512 tiles of 32 rays) fit 32 bits
-    unsigned c[kCnt];
-    for (int k = 0; k < kCnt; k++) c[k] = 0u;
-    const int kc = a.count ? kCnt : 7;  // the trace writes the traversal counters only when counting
+    // hand-offs, segments and hits of one block (at most 32768 tiles of 32 rays) fit 32 bits
+    unsigned c[kCntRay];
+    for (int k = 0; k < kCntRay; k++) c[k] = 0u;
     int mine = 0;
     for (int t = t0 + (int)threadIdx.x; t < t1; t += blockDim.x) {
         const float2 *pp = reinterpret_cast<const float2 *>(a.partials + (base + t) * 6);
@@ -3254,7 +3253,7 @@ __global__ void __launch_bounds__(32 * kRedWarps, kRedBlocksPerSM) k_reduce1(Tra
             else f32[k].hi = __fadd_rn(f32[k].hi, p);
         }
         // count 0: the tile's hand-off flags; the re-trace below counts the rays it does
-        for (int k = 1; k < kc; k++) c[k] += a.pcounts[(base + t) * kCnt + k];
+        for (int k = 1; k < kCntRay; k++) c[k] += a.pcounts[(base + t) * kCnt + k];
         mine |= a.amb_count[base + t];
     }
     __shared__ TraceCtx B;
@@ -3276,7 +3275,7 @@ __global__ void __launch_bounds__(32 * kRedWarps, kRedBlocksPerSM) k_reduce1(Tra
             else if (mode == 1) comp_add(f32[k], (float)acc[k]);
             else f32[k].hi = __fadd_rn(f32[k].hi, (float)acc[k]);
         }
-        for (int k = 0; k < kCnt; k++) c[k] += (unsigned)acc[6 + k];
+        for (int k = 0; k < kCntRay; k++) c[k] += (unsigned)acc[6 + k];
         if (flags) atomicOr(&blk_flags, flags);
         __syncthreads();
         if (threadIdx.x == 0 && blk_flags) atomicOr(&a.pose[s].flags, blk_flags);
@@ -3293,9 +3292,17 @@ __global__ void __launch_bounds__(32 * kRedWarps, kRedBlocksPerSM) k_reduce1(Tra
     } else {
         for (int k = 0; k < 6; k++) sh.r32[k][threadIdx.x] = f32[k];
     }
-    for (int k = 0; k < kCnt; k++) {
-        // only the live counts (kc is uniform over the launch)
-        const unsigned x = k < kc ? __reduce_add_sync(0xffffffffu, c[k]) : c[k];
+    for (int k = 0; k < kCntRay; k++) {
+        const unsigned x = __reduce_add_sync(0xffffffffu, c[k]);
+        if (lane == 0) rc[k][w] = x;
+    }
+    // the traversal counters, which the trace writes only when counting: thousands of nodes a ray pass 32 bits
+    for (int k = kCntRay; k < kCnt; k++) {
+        unsigned long long x = 0ull;
+        if (a.count) {
+            for (int t = t0 + (int)threadIdx.x; t < t1; t += blockDim.x) x += a.pcounts[(base + t) * kCnt + k];
+            for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        }
         if (lane == 0) rc[k][w] = x;
     }
     __syncthreads();
