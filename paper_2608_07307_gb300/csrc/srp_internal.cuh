@@ -283,18 +283,23 @@ inline size_t qstate_words(size_t slots) { return (size_t)kQSlot + 3 * slots; }
 constexpr int kFewSlots = 4;
 inline bool few_slots(int S) { return S < kFewSlots; }
 // Does k_trace_few trace the launch?  It wins where the launch waits for its
-// slowest warps, that is for few rays and long walks: the one-lane kernel's time
-// on one evaluation is 45, 58, 90, 130, 180 us of tail at 900, 3k, 12k, 50k and
-// 200k triangles (plus its throughput time), k_trace_few's 28 us plus 0.18 us per
-// 1000 rays.  Measured on single evaluations (old / few, us): 900 triangles 256^2
-// 45 / 41, 512^2 51 / 67; 3k 256^2 58 / 42, 512^2 66 / 65; 12k 512^2 90 / 70; 50k
-// 512^2 130 / 75, 777^2 (2 bounces) 224 / 146, 1024^2 157 / 162; 200k 256^2 148 /
-// 60, 512^2 184 / 87, 1024^2 (2 bounces) 332 / 219, 1448^2 284 / 318: the line
-// rays = 4000 sqrt(triangles) lies between the two everywhere.
+// slowest warps, that is for few rays and long walks; the one-lane kernel issues
+// fewer instructions and wins where the launch's rays keep the SMs busy.  Whole
+// calls, one-lane / few, us, means of eight directions:
+//   one bounce: 900 triangles 128^2 133 / 125, 256^2 148 / 146, 384^2 156 / 160;
+//   3k 256^2 143 / 133, 512^2 171 / 179; 12k 384^2 170 / 153, 512^2 179 / 171, 777^2
+//   219 / 243; 50k 512^2 193 / 169 (two of them 228 / 216, three 271 / 264), 777^2 240 /
+//   256; 200k 512^2 214 / 173 (three 353 / 298), 777^2 254 / 242, 1024^2 287 / 308;
+//   two bounces: 900 256^2 168 / 160, 512^2 185 / 193; 12k 512^2 215 / 192 (three 299 /
+//   305); 50k 512^2 239 / 193 (three 366 / 289), 1024^2 337 / 352; 200k 512^2 277 / 199,
+//   1024^2 367 / 336 (two 560 / 531).
+// The two meet near 2400 sqrt(triangles) rays with one bounce and 4600 with two,
+// whether the rays are of one slot or of three.  The line lies below, since single
+// directions differ (near it a call is up to 1.3 times as long, or half).
 inline bool few_trace(int S, size_t rays, int nseg, bool raster, int n_tris)
 {
-    const double r = (double)S * (double)rays;
-    return few_slots(S) && nseg > 1 && raster && r * r <= 1.6e7 * (double)n_tris;
+    const double r = (double)S * (double)rays / (nseg > 2 ? 2 : 1);
+    return few_slots(S) && nseg > 1 && raster && r * r <= 4.0e6 * (double)n_tris;
 }
 // k_diffuse blocks per slot (fixed: the sums have a fixed order), added in kDiffSums groups (block b in
 // group b mod kDiffSums).  Items cost very different times, and with as many blocks as run at once a
