@@ -129,7 +129,9 @@ typedef struct {
  */
 #define SRP_MAX_DIFFUSE 256
 
-#define SRP_EVAL_COUNT 1  /* gather traversal counters (slower kernel variant)        */
+#define SRP_EVAL_COUNT 1  /* gather traversal counters (slower kernel variant; launches of few
+                             evaluations are then traced by the kernel of launches of many, with the
+                             same results: the counters are that kernel's)              */
 #define SRP_EVAL_TIMING 2 /* time each phase with CUDA events on the context stream   */
 /* Primary visibility by BVH traversal of every pixel's ray instead of the
  * default rasterisation.  All primary rays of an evaluation are parallel

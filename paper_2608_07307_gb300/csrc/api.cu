@@ -806,13 +806,10 @@ srp_status eval_enqueue(srp_ctx *ctx, Mesh *m, const srp_eval_params *prm, const
     return SRP_OK;
 }
 
-// Adjoint of evaluations whose hits were recorded earlier: posing and window
-// vertices again (no trace), then the frozen-hit reverse sweep, on `st` with
-// the first lane's slots.  hits: [n][N*N][nseg] original triangle ids.
 // The counters and the error flags of a call, one block on the device: cleared by
 // one memset, read back by one copy into pinned memory, which waits for the stream.
 // (Two memsets and two copies into pageable memory, each staged and waited for by the
-// driver: 15 us more a call.)
+// driver: 15 us more a call.  The arcs, milliseconds long, read them by separate copies.)
 constexpr size_t kResultBytes = 17 * sizeof(unsigned long long);
 cudaError_t clear_results(srp_ctx *ctx, cudaStream_t st) { return cudaMemsetAsync(ctx->stats, 0, kResultBytes, st); }
 cudaError_t fetch_results(srp_ctx *ctx, cudaStream_t st)
@@ -821,6 +818,9 @@ cudaError_t fetch_results(srp_ctx *ctx, cudaStream_t st)
     return e == cudaSuccess ? cudaStreamSynchronize(st) : e;
 }
 
+// Adjoint of evaluations whose hits were recorded earlier: posing and window
+// vertices again (no trace), then the frozen-hit reverse sweep, on `st` with
+// the first lane's slots.  hits: [n][N*N][nseg] original triangle ids.
 srp_status adj_enqueue(srp_ctx *ctx, Mesh *m, const srp_eval_params *prm, const EvalPlan &pl, int n,
                        const double *d_sun, const double *d_dist, const int32_t *hits, const AdjBatch &ab,
                        cudaStream_t st, int64_t &launches)

@@ -21,8 +21,9 @@
 // autotuner), sharing one copy of the slot context.  The tiles of every slot of
 // a launch form one flat grid, so one launch can trace different meshes, grid
 // sizes and bounce counts.  The primary segment takes the raster's nearest
-// certain hit and candidates (a pixel with too many candidates, or every pixel
-// when rasterisation is off, traverses instead).  Every traversed segment walks
+// certain hit and candidates (a pixel with too many candidates, those past two where
+// the slot's list of them ran over, or every pixel when rasterisation is off, traverses
+// instead).  Every traversed segment walks
 // each part's 4-wide BVH (128 B nodes: six float4 of child boxes in SoA order,
 // the near and far planes picked by the ray's octant, and the child refs),
 // parts in the order the ray enters their root boxes, with the watertight
@@ -38,8 +39,8 @@
 // Every FP32 decision carries an error bound: when an edge function, the
 // nearest-hit comparison or the self-hit threshold is within its bound, the
 // triangle is settled in FP64 at the end of the segment (resolve64); only a ray
-// with too many such triangles is handed to the FP64 re-trace and contributes
-// nothing here.  Per hit:
+// with too many such triangles, or that hits one without an FP32 normal, is handed
+// to the FP64 re-trace and contributes nothing here.  Per hit:
 // absorbed + specular + Lambertian momentum, torque about c_ref, specular ray
 // of weight w rho_s.  Per-ray sums in FP32 (at most 1 + bounces terms), tile
 // sums by an FP32 butterfly and integer reductions, one partial per tile; the
@@ -57,7 +58,7 @@
 // up its warp.  Same decisions, same bits.
 //
 // FP64 re-trace (in k_reduce1).  A ray whose uncertain triangles overflow the
-// candidate list is re-traced from its pixel definition with FP64 rays and
+// candidate list, or whose hit has no FP32 normal, is re-traced from its pixel definition with FP64 rays and
 // vertices, the same BVH (boxes padded well beyond the FP32 rounding of the
 // ray; leaves pre-tested in FP32 with a bound, so only triangles not certainly
 // missed are tested in FP64) and the same watertight test in FP64.
@@ -69,13 +70,13 @@
 // diffuse rays) or by k_reduce, scaled by P0 / dist^2 times the pixel area.  No
 // atomics on data: results are bit-reproducible.
 //
-// k_diffuse (optional, Sec. 6.1's diffuse rays).  After the re-trace, a thread per
-// (primary ray, sample) replays the ray's specular chain in FP64 through the recorded
-// hit triangles and, at each hit with a next level, traces its sample of the K
-// cosine-weighted diffuse rays (SplitMix64 stream) in FP32 with the same error bounds
-// (walk_warp: incoherent rays, whose lanes would wait for each other), settling the
-// uncertain triangles in FP64 (settle64); its per-block FP64 sums are added by
-// k_reduce in a fixed order.
+// k_demit, k_dscan, k_diffuse (optional, Sec. 6.1's diffuse rays).  After the re-trace,
+// a thread per primary ray replays its specular chain in FP64 through the recorded hit
+// triangles and writes a record per hit that emits; the records are counted; then a
+// thread per (record, sample) traces its sample of the K cosine-weighted diffuse rays
+// (SplitMix64 stream) in FP32 with the same error bounds (walk_warp: incoherent rays,
+// whose lanes would wait for each other), settling the uncertain triangles in FP64
+// (settle64); its per-block FP64 sums are added by k_reduce in a fixed order.
 //
 // k_bvh_check (diagnostics).  One thread per part walks slot 0's 4-wide tree and counts
 // leaf references, child boxes outside their parent's and triangles outside their leaf.
@@ -1329,9 +1330,6 @@ __device__ __noinline__ Best32 resolve64_warp(const TraceCtx &B, bool want, int 
 __device__ __noinline__ Best32 resolve64(const TraceCtx &B, int N, int i, int j, int seg, const int *hpt, int hps,
                                          int skip, Cands cd, Best32 best);
 
-// One warp per block, one 32-pixel tile (tile_w x 32 / tile_w) per block; the
-// blocks of all slots form one flat grid.  Latency bound: 32 warps per SM at
-// the kernel's 64 registers (no spills).
 // ------------------------------------------------------------- raster
 // Primary visibility by rasterisation.  Every primary ray of an evaluation runs
 // along the same direction d from its pixel centre, so the nearest hit of a
@@ -1343,7 +1341,8 @@ __device__ __noinline__ Best32 resolve64(const TraceCtx &B, int N, int i, int j,
 // that minimum: uncertain edge decisions not certainly beyond it, and certain
 // hits within its depth band (what the traversal sends to its FP64
 // resolution).  The trace then settles those candidates in FP64 exactly as
-// after a traversal; a pixel with more than kPixCand of them traverses.
+// after a traversal; a pixel with more than kPixMax of them traverses, and so does
+// one with more than kPixCand where the slot's list ran over (pix_listed).
 
 struct RastView {
     const float4 *vview;
@@ -1804,7 +1803,8 @@ __device__ __forceinline__ void trace_block(const TraceArgs &a, int vb, TraceCtx
     }
     // a block without a hit or candidate (half of a window's blocks) leaves before it copies the context
     // (its warps held their slots for ~10k cycles each: headline batch 3.95 -> 3.89 ms, 100k triangles at 777^2 2.57 ->
-    // 2.51 ms, box-wing table 1.61 -> 1.57 ms)
+    // 2.51 ms, box-wing table 1.61 -> 1.57 ms; what the key read keeps alive across the copy spills: 49.0 -> 55.1 M
+    // local-memory load sectors a headline launch)
     if (!__syncthreads_or(inside && (bad || pk != ~0ull))) {
         if (tile_id >= D.tiles) return;
         const size_t tile = (size_t)s * a.n_blocks_x + tile_id;
@@ -1953,6 +1953,7 @@ __device__ __forceinline__ void trace_block(const TraceArgs &a, int vb, TraceCtx
     tile_results<COUNT>(a, s, tile_id, ray, fac, c_handoff, c_segs, c_hitbits, cn, flags);
 }
 
+// 64 registers for 32 warps an SM (212 B of spill stores and 232 B of loads; 80 registers and fewer warps: slower).
 template <bool COUNT, bool HITS>
 __global__ void __launch_bounds__(kTileRays * kTraceWarps, 32 / kTraceWarps) k_trace(TraceArgs a)
 {
@@ -2137,7 +2138,7 @@ __global__ void __launch_bounds__(32 * kFewWarps, kFewBlocksPerSM) k_trace_few(T
         // (the same for every ray of the segment: the lanes test each other's rays)
         delta = B.delta_s + 2.0f * delta;
         tau = 64.0f * delta + 32.0f * kU * (B.R + B.L);
-        // ---- every warp: the walks of every fourth ray
+        // ---- every warp: the walks of its share, every kFewWarps-th ray
         if (w < n) {
             const int at = w + kFewWarps * lane;
             const bool mine = at < n;
@@ -2962,16 +2963,12 @@ __device__ __forceinline__ void diffuse_sample(const TraceCtx &B, WalkShared &S,
     acc[5] += arm[0] * F[1] - arm[1] * F[0];
 }
 
-// Diffuse secondary rays of every ray of slot s (grid: kDiffBlocks x slots; a
-// thread per (primary ray, sample q) work item in turn, so the K lanes of one
-// ray share its control flow).  The ray's segments are replayed in FP64
-// through the triangles the trace recorded (hit point on the triangle's
-// plane, specular direction), and at each hit of a segment with a next level
-// sample q of the K rays of weight w rho_d / K, cosine-distributed about the
-// lit side's normal, is traced with the FP64 traversal and deposits the
-// per-hit law at its hit.  Sums per block in a fixed order: the result is
+// Diffuse secondary rays of slot s, in three launches of kDiffBlocks blocks (k_dscan:
+// one) a slot: the hits that emit (segments with a next level), their number, and K rays
+// a hit of weight w rho_d / K, cosine-distributed about the lit side's normal, which
+// deposit the per-hit law at theirs.  Sums per block in a fixed order: the result is
 // reproducible.
-// Diffuse rays, step 1: a thread per primary ray replays its specular chain in
+// Step 1: a thread per primary ray replays its specular chain in
 // FP64 through the recorded hit triangles and writes one record per hit that
 // emits (a segment with a next level, rho_d > 0) to the ray's slots of the
 // dense array, and the number of records.
@@ -3036,7 +3033,7 @@ __global__ void __launch_bounds__(kLaneStride) k_demit(TraceArgs a)
     }
 }
 
-// Diffuse rays, step 2: a block per slot turns the per-ray record counts into
+// Step 2: a block per slot turns the per-ray record counts into
 // their exclusive prefix (each thread a contiguous range, then the block's
 // ranges in order) and the slot's total.
 __global__ void __launch_bounds__(1024) k_dscan(TraceArgs a)
@@ -3067,10 +3064,11 @@ __global__ void __launch_bounds__(1024) k_dscan(TraceArgs a)
     if (threadIdx.x == blockDim.x - 1) a.dtot[s] = part[threadIdx.x];
 }
 
-// Diffuse rays, step 3: a thread per (record, sample) work item, items in the
+// Step 3: a thread per (record, sample) work item, items in the
 // order of the records (ray-major), each record's K samples consecutive; the
 // record of item e K + q is found by binary search over the prefix.
-// (four blocks an SM, 128 registers: 3.08 ms against 3.57 at three and 3.50 at five, at 64 blocks a slot)
+// (four blocks an SM, 128 registers, 144 B of spills: 3.08 ms against 3.57 at three and 3.50 at five, at 64 blocks a
+// slot)
 __global__ void __launch_bounds__(kLaneStride, 4) k_diffuse(TraceArgs a)
 {
     pdl_enter();
@@ -3144,7 +3142,7 @@ __device__ void final_reduce(const TraceArgs &a, int s, int eval0, double *force
 // up to 32 of them run at once: the two meet near four rays a warp.
 constexpr int kWarpRays = 32;
 // Warps of a first-level block, resident blocks: 32 box-wing evaluations a launch 39 us at two
-// blocks an SM (128 registers), 32.6 at four (the re-trace spills, rarely run), 31.6 at five.
+// blocks an SM (128 registers), 32.6 at four (the re-trace, rarely run, spills 372 B), 31.6 at five.
 constexpr int kRedWarps = 8, kRedBlocksPerSM = 4;
 
 struct RefineShared {
