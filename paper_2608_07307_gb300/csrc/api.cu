@@ -1420,6 +1420,8 @@ srp_status srp_mesh_load(srp_ctx *ctx, const srp_mesh_desc *D, int32_t *mesh_id)
     MK(cudaMemsetAsync(cnt_static, 0, sizeof(unsigned) * std::max(h.n_static_nodes, 1), st));
     // device copy of the mesh, then the static refit (writes root boxes into it)
     MK(dmalloc(m->allocs, &m->d, 1));
+    for (int p = 0; p < NP; p++)
+        for (int k = 0; k < 6; k++) h.root_box_static[p][k] = h.part[p].tri_count > 0 ? 0.f : INFINITY;
     MK(cudaMemcpyAsync(m->d, &h, sizeof(MeshDev), cudaMemcpyHostToDevice, st));
     MK(launch_refit_static(m->d, h, h.node_static, h.tri_static, cnt_static, &m->d->root_box_static[0][0], st));
     MK(cudaMemcpyAsync(&h.root_box_static[0][0], &m->d->root_box_static[0][0], sizeof(h.root_box_static),

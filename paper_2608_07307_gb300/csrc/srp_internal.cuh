@@ -175,7 +175,7 @@ struct MeshDev {
                            // plus the posing error bound, metres)
     float2 *mat32;         // [n_mats] (rho_s, rho_d) FP32
     double *mat64;         // [n_mats][2]
-    float root_box_static[kMaxParts][6];
+    float root_box_static[kMaxParts][6];  // (of a part without triangles: all six +inf, which no ray enters)
 };
 
 // Per-slot dynamic storage (one block of arrays per concurrent evaluation).

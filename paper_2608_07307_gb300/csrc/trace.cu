@@ -105,7 +105,7 @@ struct PartView {
     int limit;           // bound on loop iterations of one part walk (nodes + triangles)
     int tri_begin, vert_begin;
     float box[6];        // root box (filled when a block loads the context, from box_src)
-    const float *box_src;  // the part's root box: the refit's output for a dynamic part
+    const float *box_src;  // the part's root box: the refit's output for a dynamic part with triangles
 };
 
 struct TraceCtx {
@@ -246,7 +246,7 @@ __global__ void k_frame(TraceArgs a)
         pv.tri_begin = pi.tri_begin;
         pv.vert_begin = pi.vert_begin;
         pv.v4 = tri_v4 + pi.tri_begin;
-        if (pi.dynamic) {
+        if (pi.dynamic && pi.tri_count > 0) {
             pv.node = sb.node + (size_t)pi.dyn_node_off * kNode4;
             pv.tri = sb.tri + (size_t)pi.dyn_tri_off * 3;
             pv.v64 = sb.vert64 + (size_t)pi.dyn_vert_off * 3;
@@ -3443,7 +3443,7 @@ __global__ void k_bvh_check(const unsigned char *tctx, int *tri_seen, unsigned l
 {
     const TraceCtx &B = *reinterpret_cast<const TraceCtx *>(tctx);
     const PartView &pv = B.part[blockIdx.x];
-    if (threadIdx.x != 0) return;
+    if (threadIdx.x != 0 || !(pv.box_src[0] < INFINITY)) return;  // (a part without triangles)
     unsigned long long refs = 0, outside_box = 0, outside_tri = 0, nodes = 0, bound = 0;
     auto inside = [](const float *in, const float *out) {
         return in[0] >= out[0] && in[1] <= out[1] && in[2] >= out[2] && in[3] <= out[3] && in[4] >= out[4] &&
